@@ -43,6 +43,27 @@ def test_transpose_long_columns(sg):
     assert np.array_equal(val, R.val)
 
 
+@pytest.mark.parametrize("m", [9000, 460_000, 2_200_000])
+@pytest.mark.parametrize("index", [np.int32, np.int64])
+def test_transpose_column_lengths(sg, m, index):
+    # column lengths at the edges of the row sorts of A^T (8 lanes, a warp's
+    # registers, a warp's shared memory, a block) and of the bitmap's windows
+    # (458752 rows): 9000 rows fit one, 2.2 M take five; there, columns of up
+    # to 1074 entries are too sparse for the bitmap and take the bitonic sort
+    rng = np.random.default_rng(m)
+    lens = [0, 1, 7, 8, 9, 31, 32, 33, 63, 64, 65, 255, 256, 257, 1073, 1074, 1075, 8191, 8192,
+            8193, 8999]
+    lens = np.array(lens + [3] * 40 + lens[::-1])
+    rows = np.concatenate([rng.choice(m, size=k, replace=False) for k in lens])
+    cols = np.repeat(np.arange(lens.size), lens)
+    A = inputs.coo_to_csr(m, lens.size, rows, cols, rng.random(rows.size), index)
+    T = sg.transpose(sg.to_device(A))
+    rp, col, val = T.to_host()
+    R = oracle.transpose(A)
+    assert np.array_equal(rp, R.rowptr) and np.array_equal(col, R.col)
+    assert np.array_equal(val, R.val)
+
+
 def small_batch(value="u11_f32", count=24, seed=3):
     rng = np.random.default_rng(seed)
     out = []
