@@ -22,6 +22,7 @@
 #include <cstdio>
 
 #include "plan.h"
+#include "rows.cuh"
 
 namespace sg {
 
@@ -72,29 +73,43 @@ __global__ void final_counts_kernel(long long R, const int64_t* __restrict__ slo
     }
 }
 
-// Compaction: one warp per row copies it from its slot or from the re-run.
+// Compaction: every row is copied from its slot or from the re-run (four
+// entries per lane in flight; a block for the longest rows).
 template <class IT, class V>
-__global__ void compact_kernel(long long R, const int64_t* __restrict__ slots,
-                               const int32_t* __restrict__ inv, const int64_t* __restrict__ rp_x,
-                               const IT* __restrict__ col_s, const V* __restrict__ val_s,
-                               const IT* __restrict__ col_x, const V* __restrict__ val_x,
-                               const int64_t* __restrict__ rp_f, IT* __restrict__ col_f,
-                               V* __restrict__ val_f) {
-    const int lane = lane_id();
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long r = warp; r < R; r += nwarps) {
-        const int t = inv[r];
-        const long long src = t >= 0 ? rp_x[t] : slots[r];
-        const IT* cs = t >= 0 ? col_x : col_s;
-        const V* vs = t >= 0 ? val_x : val_s;
-        const long long dst = rp_f[r];
-        const long long L = rp_f[r + 1] - dst;
-        for (long long q = lane; q < L; q += 32) {
-            col_f[dst + q] = cs[src + q];
-            if constexpr (VOps<V>::has_val) val_f[dst + q] = vs[src + q];
-        }
-    }
+__global__ void __launch_bounds__(kRowWarps * 32)
+    compact_kernel(long long R, const int64_t* __restrict__ slots,
+                   const int32_t* __restrict__ inv, const int64_t* __restrict__ rp_x,
+                   const IT* __restrict__ col_s, const V* __restrict__ val_s,
+                   const IT* __restrict__ col_x, const V* __restrict__ val_x,
+                   const int64_t* __restrict__ rp_f, IT* __restrict__ col_f,
+                   V* __restrict__ val_f) {
+    for_rows(
+        R, 2048, [&](long long r) { return rp_f[r + 1] - rp_f[r]; },
+        [&](long long r, int w, auto warps) {
+            constexpr int stride = 32 * decltype(warps)::value;
+            const int t = inv[r];
+            const long long src = t >= 0 ? rp_x[t] : slots[r];
+            const IT* cs = (t >= 0 ? col_x : col_s) + src;
+            const V* vs = (t >= 0 ? val_x : val_s) + src;
+            const long long dst = rp_f[r];
+            const long long L = rp_f[r + 1] - dst;
+            for (long long q = 32 * w + lane_id(); q < L; q += 4 * stride) {
+                IT c[4];
+                V v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (q + u * stride < L) {
+                        c[u] = cs[q + u * stride];
+                        v[u] = load_val(vs, q + u * stride);
+                    }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (q + u * stride < L) {
+                        col_f[dst + q + u * stride] = c[u];
+                        if constexpr (VOps<V>::has_val) val_f[dst + q + u * stride] = v[u];
+                    }
+            }
+        });
 }
 
 template <class IT, class V>
@@ -104,7 +119,7 @@ cudaError_t launch_compact(long long R, int sms, cudaStream_t s, const int64_t* 
                            const int64_t* rp_f, void* col_f, void* val_f) {
     const unsigned g = (unsigned)std::max<long long>(1, std::min<long long>((R + 7) / 8, (long long)sms * 8));
     count_launches(1);
-    compact_kernel<IT, V><<<g, 256, 0, s>>>(R, slots, inv, rp_x, (const IT*)col_s, (const V*)val_s,
+    compact_kernel<IT, V><<<g, kRowWarps * 32, 0, s>>>(R, slots, inv, rp_x, (const IT*)col_s, (const V*)val_s,
                                             (const IT*)col_x, (const V*)val_x, rp_f, (IT*)col_f,
                                             (V*)val_f);
     return cudaGetLastError();

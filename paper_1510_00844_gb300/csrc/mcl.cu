@@ -3,69 +3,130 @@
 // of M^T are the columns of M), drop every entry below `threshold` and divide
 // each row by the sum of its kept entries, so M stays column-stochastic.
 // Input may be a view (rowend); output is a plain CSR of float64 values.
-// Pass 1 (one warp per row): kept count and kept sum; scan; pass 2: the kept
-// entries, in order, divided by the row sum.  The sum of a row is a warp
-// reduction over its kept entries in a fixed order, so results repeat
-// exactly from run to run.
+// Pass 1: kept count and kept sum per row; scan; pass 2: the kept entries, in
+// order, divided by the row sum.  A row's sum is formed in an order that its
+// length alone fixes (a warp's lanes side by side, or a block's threads for a
+// row of more than kMclLong entries), so results repeat exactly from run to
+// run and do not depend on how the row is stored.
+// What bounds it: the FP64 pipe, which a warp's compare, add or (ten
+// instructions) division takes however many lanes are active.  So values are
+// compared as integers, and divided after they have been compacted, 32 at a
+// time.  R-MAT, 40009 vertices (87 M entries, rows up to 23467): count 0.51 ->
+// 0.31 ms, fill 2.33 -> 0.80 ms (a warp per row, one load in flight per lane, and
+// divisions where the kept entries stood).
 #include <cstdio>
 
 #include "plan.h"
+#include "rows.cuh"
 
 namespace sg {
 
-template <class IT>
-__global__ void mcl_count_kernel(long long m, const int64_t* __restrict__ rp,
-                                 const int64_t* __restrict__ re, const double* __restrict__ val,
-                                 double thr, int64_t* __restrict__ cnt, double* __restrict__ sums) {
-    const int lane = lane_id();
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long i = warp; i < m; i += nwarps) {
-        const long long a = rp[i], b = re ? re[i] : rp[i + 1];
-        long long c = 0;
-        double s = 0.0;
-        for (long long q = a + lane; q < b; q += 32) {
-            const double v = val[q];
-            if (v >= thr) {
-                ++c;
-                s = __dadd_rn(s, v);
-            }
+constexpr long long kMclLong = 2048;
+
+// v >= threshold without the FP64 pipe: for a positive threshold the bits of
+// doubles compare like integers (negative values below, NaN above infinity).
+struct AtLeast {
+    double threshold;
+    __device__ __forceinline__ bool operator()(double v) const {
+        if (__double_as_longlong(threshold) > 0) {
+            const long long b = __double_as_longlong(v);
+            return b >= __double_as_longlong(threshold) && b <= 0x7ff0000000000000LL;
         }
-        c = warp_sum(c);
-#pragma unroll
-        for (int d = 16; d; d >>= 1) s = __dadd_rn(s, __shfl_xor_sync(kFull, s, d));
-        if (lane == 0) {
-            cnt[i] = c;
-            sums[i] = s;
-        }
+        return v >= threshold;
     }
+};
+
+__global__ void __launch_bounds__(kRowWarps * 32)
+    mcl_count_kernel(long long m, const int64_t* __restrict__ rp, const int64_t* __restrict__ re,
+                     const double* __restrict__ val, double thr, int64_t* __restrict__ cnt,
+                     double* __restrict__ sums) {
+    const AtLeast keeps{thr};
+    __shared__ long long part_c[kRowWarps];
+    __shared__ double part_s[kRowWarps];
+    for_rows(
+        m, kMclLong, [&](long long i) { return (re ? re[i] : rp[i + 1]) - rp[i]; },
+        [&](long long i, int w, auto warps) {
+            constexpr int WARPS = decltype(warps)::value;
+            constexpr int stride = 32 * WARPS;
+            const long long a = rp[i], b = re ? re[i] : rp[i + 1];
+            long long c = 0;
+            double s = 0.0;
+            for (long long q0 = a + 32 * w + lane_id(); q0 < b; q0 += 4 * stride) {
+                double v[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = q0 + u * stride < b ? val[q0 + u * stride] : 0.0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (q0 + u * stride < b && keeps(v[u])) {
+                        ++c;
+                        s = __dadd_rn(s, v[u]);
+                    }
+            }
+            c = warp_sum(c);
+#pragma unroll
+            for (int d = 16; d; d >>= 1) s = __dadd_rn(s, __shfl_xor_sync(kFull, s, d));
+            if constexpr (WARPS > 1) {
+                if (lane_id() == 0) {
+                    part_c[w] = c;
+                    part_s[w] = s;
+                }
+                __syncthreads();
+                c = 0;
+                s = 0.0;
+                for (int t = 0; t < WARPS; ++t) {
+                    c += part_c[t];
+                    s = __dadd_rn(s, part_s[t]);
+                }
+            }
+            if (w == 0 && lane_id() == 0) {
+                cnt[i] = c;
+                sums[i] = s;
+            }
+        });
 }
 
 template <class IT>
-__global__ void mcl_fill_kernel(long long m, const int64_t* __restrict__ rp,
-                                const int64_t* __restrict__ re, const IT* __restrict__ col,
-                                const double* __restrict__ val, double thr,
-                                const double* __restrict__ sums, const int64_t* __restrict__ rpo,
-                                IT* __restrict__ colo, double* __restrict__ valo) {
-    const int lane = lane_id();
-    const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long i = warp; i < m; i += nwarps) {
-        const long long a = rp[i], b = re ? re[i] : rp[i + 1];
-        long long out = rpo[i];
-        const double s = sums[i];
-        for (long long q0 = a; q0 < b; q0 += 32) {
-            const long long q = q0 + lane;
-            const bool keep = q < b && val[q] >= thr;
-            const unsigned msk = __ballot_sync(kFull, keep);
-            if (keep) {
-                const long long pos = out + __popc(msk & lanemask_lt());
-                colo[pos] = col[q];
-                valo[pos] = __ddiv_rn(val[q], s);
+__global__ void __launch_bounds__(kRowWarps * 32)
+    mcl_fill_kernel(long long m, const int64_t* __restrict__ rp, const int64_t* __restrict__ re,
+                    const IT* __restrict__ col, const double* __restrict__ val, double thr,
+                    const double* __restrict__ sums, const int64_t* __restrict__ rpo,
+                    IT* __restrict__ colo, double* valo) {
+    const AtLeast keeps{thr};
+    for_rows(
+        m, kMclLong, [&](long long i) { return (re ? re[i] : rp[i + 1]) - rp[i]; },
+        [&](long long i, int w, auto warps) {
+            const long long a = rp[i], n = (re ? re[i] : rp[i + 1]) - a, out = rpo[i];
+            const double s = sums[i];
+            constexpr int WARPS = decltype(warps)::value;
+            constexpr int wide = 32 * WARPS;
+            double v[4];
+            long long at[4];
+            filter_entries<WARPS>(
+                n, w,
+                [&](long long q, int stride) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        at[u] = a + q + u * stride;
+                        v[u] = q + u * stride < n ? val[at[u]] : 0.0;
+                    }
+                },
+                [&](int u) { return keeps(v[u]); },
+                [&](int u, long long pos) {
+                    colo[out + pos] = col[at[u]];
+                    valo[out + pos] = v[u];
+                });
+            if constexpr (WARPS > 1) __syncthreads();
+            else __syncwarp();
+            // the row's kept values, now side by side
+            const long long end = rpo[i + 1];
+            for (long long q = out + 32 * w + lane_id(); q < end; q += 4 * wide) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) v[u] = q + u * wide < end ? valo[q + u * wide] : 1.0;
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (q + u * wide < end) valo[q + u * wide] = __ddiv_rn(v[u], s);
             }
-            out += __popc(msk);
-        }
-    }
+        });
 }
 
 }  // namespace sg
@@ -114,12 +175,9 @@ spgemm_status spgemm_mcl_prune_count(const spgemm_csr* C, double threshold, void
     if (e == cudaSuccess && m > 0) {
         const unsigned g = (unsigned)std::max<long long>(1, std::min<long long>((m + 7) / 8, (long long)sms * 8));
         sg::count_launches(1);
-        if (C->index_type == SPGEMM_INDEX_I32)
-            sg::mcl_count_kernel<int32_t><<<g, 256, 0, s>>>(m, C->rowptr, C->rowend, (const double*)C->val,
-                                                            threshold, rowptrP, sums);
-        else
-            sg::mcl_count_kernel<int64_t><<<g, 256, 0, s>>>(m, C->rowptr, C->rowend, (const double*)C->val,
-                                                            threshold, rowptrP, sums);
+        sg::mcl_count_kernel<<<g, sg::kRowWarps * 32, 0, s>>>(m, C->rowptr, C->rowend,
+                                                              (const double*)C->val, threshold,
+                                                              rowptrP, sums);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = sg::launch_exclusive_scan(rowptrP, m + 1, temp, s);
@@ -148,11 +206,11 @@ spgemm_status spgemm_mcl_prune_fill(const spgemm_csr* C, double threshold, void*
     const unsigned g = (unsigned)std::max<long long>(1, std::min<long long>((m + 7) / 8, (long long)sms * 8));
     sg::count_launches(1);
     if (C->index_type == SPGEMM_INDEX_I32)
-        sg::mcl_fill_kernel<int32_t><<<g, 256, 0, s>>>(m, C->rowptr, C->rowend, (const int32_t*)C->col,
+        sg::mcl_fill_kernel<int32_t><<<g, sg::kRowWarps * 32, 0, s>>>(m, C->rowptr, C->rowend, (const int32_t*)C->col,
                                                        (const double*)C->val, threshold, (const double*)ws,
                                                        rowptrP, (int32_t*)colP, valP);
     else
-        sg::mcl_fill_kernel<int64_t><<<g, 256, 0, s>>>(m, C->rowptr, C->rowend, (const int64_t*)C->col,
+        sg::mcl_fill_kernel<int64_t><<<g, sg::kRowWarps * 32, 0, s>>>(m, C->rowptr, C->rowend, (const int64_t*)C->col,
                                                        (const double*)C->val, threshold, (const double*)ws,
                                                        rowptrP, (int64_t*)colP, valP);
     cudaError_t e = cudaGetLastError();

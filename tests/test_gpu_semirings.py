@@ -97,3 +97,25 @@ def test_masked_products(sg, complement, sr):
     name = {0: "plus_times", 2: "min_plus", 3: "min_select2nd"}[sr]
     R = oracle.mask(oracle.spgemm(A, A, semiring=name), M, complement)
     assert_equal_host(C, R)
+
+
+@pytest.mark.parametrize("complement", [False, True])
+@pytest.mark.parametrize("index", [np.int32, np.int64])
+def test_mask_row_lengths(sg, complement, index):
+    # either side the shorter one; walked lists at the edges of a warp's step
+    # (128 entries), of the rows a block takes (beyond 512) and of its step (1024)
+    rng = np.random.default_rng(92)
+    sizes = [0, 1, 31, 32, 33, 127, 128, 129, 511, 512, 513, 1023, 1024, 1025, 3000]
+    pairs = [(a, b) for a in sizes for b in (0, 1, 128, 513, 1500, 4000)]
+    n = 5000
+
+    def rows(lens, seed):
+        r = np.random.default_rng(seed)
+        col = [np.sort(r.choice(n, k, replace=False)) for k in lens]
+        rowptr = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+        col = np.concatenate(col).astype(index)
+        return inputs.CSR(len(lens), n, rowptr, col, r.integers(-9, 9, col.size))
+
+    C, M = rows([a for a, _ in pairs], 93), rows([b for _, b in pairs], 94)
+    P = sg.mask(sg.to_device(C), sg.to_device(M.pattern()), complement)
+    assert_equal_host(P, oracle.mask(C, M.pattern(), complement))
