@@ -120,7 +120,7 @@ typedef struct {
                                 nonzero stages every list's entries in shared memory with
                                 bulk asynchronous copies (cp.async.bulk, mbarrier waits bounded,
                                 SPGEMM_ERR_TIMEOUT from spgemm_merge_check if one expires);
-                                0 keeps register windows (measured faster on GB300) */
+                                0 merges through a column map (measured faster on GB300) */
 } spgemm_opts;
 
 typedef struct spgemm_plan_s* spgemm_plan_t;
@@ -481,10 +481,9 @@ size_t spgemm_merge_workspace_size(int32_t c, int64_t m, int64_t n);
 
 /* spgemm_merge_symbolic -- parts[0..c-1]: c partial products of equal shape
  * (sorted rows).  Writes rowptrC (int64[m+1]) of C = sum_s parts[s] and
- * nnz(C) (host).  Waits for the stream.  Performance only: with c <= 4 and
- * int32 column arrays whose addresses are multiples of 16 bytes, the count
- * reads four columns per lane per load; each part's nnz must then be the
- * length of its col array (as stated for spgemm_csr). */
+ * nnz(C) (host).  Waits for the stream.  Each part's nnz must be the length of its
+ * col array (as stated for spgemm_csr): a row of more than 8192 entries over
+ * all parts is cut into segments only if they can hold that many. */
 spgemm_status spgemm_merge_symbolic(int32_t c, const spgemm_csr* parts, const spgemm_opts* opts,
                                     void* stream, void* ws, size_t ws_bytes, int64_t* rowptrC,
                                     int64_t* nnz_c);

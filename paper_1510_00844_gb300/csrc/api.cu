@@ -611,7 +611,8 @@ size_t spgemm_merge_workspace_size(int32_t c, int64_t m, int64_t n) {
     (void)c;
     (void)n;
     if (m < 0) m = 0;
-    return align_up(sizeof(sg::DevCounters)) + align_up(sg::scan_temp_bytes(m + 1));
+    return align_up(sizeof(sg::DevCounters)) + align_up(sg::scan_temp_bytes(m + 1)) +
+           align_up(sizeof(sg::MergeLong));
 }
 
 
@@ -636,7 +637,9 @@ spgemm_status spgemm_merge_symbolic(int32_t c, const spgemm_csr* parts, const sp
     SG_CUDA(cudaMemsetAsync(cnt, 0, sizeof(sg::DevCounters), s), "merge: memset");
     SG_CUDA(cudaMemsetAsync(rowptrC + m, 0, sizeof(int64_t), s), "merge: memset");
     cudaError_t e = sg::launch_merge(c, parts, vt, m, n, sms, s, false, rowptrC, nullptr, nullptr,
-                                     nullptr, &cnt->err, &cnt->work_counter[0]);
+                                     nullptr, &cnt->err, &cnt->work_counter[0],
+                                     (sg::MergeLong*)((unsigned char*)temp +
+                                                      align_up(sg::scan_temp_bytes(m + 1))));
     if (e != cudaSuccess) return cuda_fail(e, "merge symbolic");
     e = sg::launch_exclusive_scan(rowptrC, m + 1, temp, s);
     if (e != cudaSuccess) return cuda_fail(e, "merge symbolic: scan");
@@ -670,6 +673,9 @@ spgemm_status spgemm_merge_numeric(int32_t c, const spgemm_csr* parts, const spg
     const bool staged = opts && opts->merge_staged;
     cudaError_t e = sg::launch_merge(c, parts, vt, m, n, sms, (cudaStream_t)stream, true, nullptr,
                                      rowptrC, colC, valC, &cnt->err, &cnt->work_counter[1],
+                                     (sg::MergeLong*)((unsigned char*)ws +
+                                                      align_up(sizeof(sg::DevCounters)) +
+                                                      align_up(sg::scan_temp_bytes(m + 1))),
                                      staged);
     if (e != cudaSuccess) return cuda_fail(e, "merge numeric");
     return SPGEMM_OK;

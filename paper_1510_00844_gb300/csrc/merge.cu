@@ -2,16 +2,27 @@
 // ascending s: the result of the paper's multiway merge with duplicate
 // reduction (Sec. 4.3), used for the LocalMerge of the k-slice partials
 // (Alg. 2).  The paper merges sorted triple lists with a heap of size c; here
-// one warp owns a row and sweeps its column range in chunks of W columns: for
-// each chunk it streams the chunk's part of every list in order s = 0..c-1
-// (a list has distinct columns, so one round never repeats a slot) into a
-// dense accumulator with a presence bitmap, then emits the chunk in column
-// order.  Chunks no list touches are skipped by jumping to the smallest next
-// column over the c cursors (lane s holds the cursor of list s).  Up to eight
-// lists take merge_win_kernel, which keeps every list's next entries in
-// flight; more lists take merge_kernel.  The count pass of up to four int32
-// lists in 16-byte aligned arrays takes merge_count4_kernel (four columns
-// per lane per load).
+// one warp owns a row (or a column segment of a long one) and takes it in
+// chunks of at most S entries over all lists: each list offers a share of the
+// next S entries in proportion to what it has left, and the chunk ends at the
+// smallest column that a list could not offer.  The chunk's columns set bits
+// in a column map; the bits before a column are its place among the chunk's
+// outputs, so the accumulator holds outputs and not columns.  The lists' values
+// are then added in order s = 0..c-1 (a list has distinct columns, so 32 of
+// its entries never repeat a place) and the chunk is written, all lanes side
+// by side.
+//
+// Rows of more than kMergeLong entries are listed and cut into kMergeSegs
+// column segments: a power-law graph's longest row holds more entries than a
+// warp should add while the others have finished.
+//
+// What bounds it: the latency of a chunk's few dependent steps (columns, map,
+// values) at 20 warps per SM, then DRAM.  The sweep of 1024-column chunks that
+// this replaces met few entries per chunk on rows of ordinary length and left
+// the longest rows to single warps.  Before and now: four lists of 100003-vertex
+// R-MAT graphs (3.3 GB read and written) 5.70 and 2.90 ms; the four partial
+// products of a 65536-vertex graph squared (11 GB) 8.9 and 7.3 ms; nine
+// partial products 40.6 and 13.4 ms.
 #include <type_traits>
 
 #include "plan.h"
@@ -19,6 +30,14 @@
 namespace sg {
 
 constexpr int kMaxMergeParts = 32;
+constexpr int kMergeWarps = 4;
+// Columns a chunk may span, and the most entries it takes: the numeric pass
+// holds an accumulator and two 16-bit columns per entry, the count only bits.
+// More of either costs warps: twice the span 2.8 and 7.9 ms, twice the span
+// and the entries 3.2 and 8.8 ms for the first two figures above.
+constexpr int kMergeSpan = 16384;
+constexpr int kMergeS = 512;
+constexpr int kMergeCountS = 2048;
 
 template <class IT, class V>
 struct MergeParts {
@@ -29,246 +48,320 @@ struct MergeParts {
     long long len[kMaxMergeParts];  // length of col/val of part s
 };
 
-template <class IT, class V, int W, int WARPS, bool NUMERIC>
-__global__ void __launch_bounds__(WARPS * 32)
-    merge_kernel(int c, MergeParts<IT, V> parts, long long m, long long n,
-                 int64_t* __restrict__ rowcnt, const int64_t* __restrict__ rpC,
-                 IT* __restrict__ ciC, V* __restrict__ vC, int* err) {
-    constexpr bool HV = NUMERIC && VOps<V>::has_val;
-    constexpr int NWORDS = W / 32;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int lane = lane_id();
-    const int w = threadIdx.x >> 5;
-    constexpr size_t vbytes = HV ? sizeof(V) * W : 0;
-    unsigned char* base = smem_raw + (size_t)w * (vbytes + W / 8);
-    V* acc = reinterpret_cast<V*>(base);
-    unsigned* bm = reinterpret_cast<unsigned*>(base + vbytes);
-    for (int s = lane; s < W; s += 32)
-        if constexpr (HV) acc[s] = VOps<V>::init();
-    for (int t = lane; t < NWORDS; t += 32) bm[t] = 0u;
-    __syncwarp();
-    const long long gw = (long long)blockIdx.x * WARPS + w;
-    const long long nw = (long long)gridDim.x * WARPS;
-    for (long long i = gw; i < m; i += nw) {
-        long long cur = 0, end = 0;
-        if (lane < c) {
-            cur = parts.rp[lane][i];
-            end = parts.re[lane] ? parts.re[lane][i] : parts.rp[lane][i + 1];
-        }
-        long long out = NUMERIC ? rpC[i] : 0;
-        const long long out_end = NUMERIC ? rpC[i + 1] : 0;
-        long long count = 0;
-        while (true) {
-            long long nxt = (lane < c && cur < end) ? (long long)parts.col[lane][cur] : n;
-            nxt = -warp_max(-nxt);  // warp min
-            if (nxt >= n) break;
-            const long long c0 = (nxt / W) * W;
-            const long long c1 = min(c0 + (long long)W, n);
-            for (int s = 0; s < c; ++s) {
-                long long q0 = __shfl_sync(kFull, cur, s);
-                const long long qe = __shfl_sync(kFull, end, s);
-                const IT* col = parts.col[s];
-                const V* val = parts.val[s];
-                while (q0 < qe) {
-                    long long q = q0 + lane;
-                    bool valid = q < qe;
-                    long long j = valid ? (long long)col[q] : c1;
-                    valid = valid && j < c1;
-                    int slot = (int)(j - c0);
-                    if (valid) {
-                        atomicOr(&bm[slot >> 5], 1u << (slot & 31));
-                        if constexpr (HV) acc[slot] = VOps<V>::add(acc[slot], val[q]);
-                    }
-                    __syncwarp();
-                    int got = __popc(__ballot_sync(kFull, valid));
-                    q0 += got;
-                    if (got < 32) break;
-                }
-                if (lane == s) cur = q0;
-            }
-            __syncwarp();
-            // emit (numeric) or count (symbolic) the chunk, clearing it
-            for (int t0 = 0; t0 < NWORDS; t0 += 32) {
-                const int t = t0 + lane;
-                unsigned word = t < NWORDS ? bm[t] : 0u;
-                int pc = __popc(word);
-                int incl = warp_incl_scan(pc);
-                int tot = __shfl_sync(kFull, incl, 31);
-                if constexpr (NUMERIC) {
-                    long long pos = out + incl - pc;
-                    while (word) {
-                        int b = __ffs(word) - 1;
-                        word &= word - 1;
-                        int slot = t * 32 + b;
-                        if (pos < out_end) {
-                            ciC[pos] = (IT)(c0 + slot);
-                            if constexpr (HV) vC[pos] = acc[slot];
-                        }
-                        if constexpr (HV) acc[slot] = VOps<V>::init();
-                        ++pos;
-                    }
-                }
-                if (t < NWORDS) bm[t] = 0u;
-                out += tot;
-                count += tot;
-            }
-            __syncwarp();
-        }
-        if constexpr (!NUMERIC) {
-            if (lane == 0) rowcnt[i] = count;
-        } else {
-            if (lane == 0 && out != out_end) atomicExch(err, (int)kDevCountMismatch);
-        }
-    }
-}
-
-// The same sum for c <= CM lists with the loads of every list in flight
-// together.  Each list keeps three windows of 32 consecutive entries in
-// registers (lane x holds entry x of each): the window being consumed and
-// the next two; when a window is used up the one after the last is loaded,
-// so a list's next entries arrive while the current ones are accumulated.
-// Entries are consumed in column order chunk by chunk: the entries of list s
-// inside the chunk are a prefix of what is left of its window (columns
-// ascend), so one ballot per list and window step covers them.  Rows are
-// taken from a counter; the count pass only adds up the row's columns.
+// (+, x) stores the first list's values instead of adding them to the identity.
 template <class V>
 constexpr bool kStoreFirst = std::is_same<V, double>::value || std::is_same<V, float>::value ||
                              std::is_same<V, int64_t>::value;
 
-template <class IT, class V, int W, int WARPS, bool NUMERIC, int CM>
-__global__ void __launch_bounds__(WARPS * 32)
-    merge_win_kernel(int c, MergeParts<IT, V> parts, long long m, long long n,
-                     int64_t* __restrict__ rowcnt, const int64_t* __restrict__ rpC,
-                     IT* __restrict__ ciC, V* __restrict__ vC, int* err,
-                     unsigned long long* work) {
+// Shared memory of a warp: accumulators, the column map (bits, and for the
+// numeric pass the outputs before each word), the chunk's columns in list
+// order and in output order (offsets from its first column).
+template <class V, bool NUMERIC>
+struct MergeWarp {
+    static constexpr int kWords = kMergeSpan / 32;
+    static constexpr int kS = NUMERIC ? kMergeS : kMergeCountS;
+    static constexpr size_t kBitsAt = NUMERIC && VOps<V>::has_val ? sizeof(V) * kS : 0;
+    static constexpr size_t kBeforeAt = kBitsAt + sizeof(unsigned) * kWords;
+    static constexpr size_t kListAt = kBeforeAt + (NUMERIC ? sizeof(unsigned short) * kWords : 0);
+    static constexpr size_t kOutAt = kListAt + (NUMERIC ? sizeof(unsigned short) * kS : 0);
+    static constexpr size_t kBytes = kOutAt + (NUMERIC ? sizeof(unsigned short) * kS : 0);
+};
+
+// One row's (or segment's) merge by a warp: lane s holds list s's range
+// [cur, end).  Returns the number of outputs; writes them from `out` on
+// (numeric; never at or past out_end).
+template <class IT, class V, bool NUMERIC>
+__device__ __forceinline__ long long merge_range(int c, const MergeParts<IT, V>& parts,
+                                                 long long cur, long long end, long long out,
+                                                 long long out_end, IT* __restrict__ ciC,
+                                                 V* __restrict__ vC, unsigned char* smem) {
+    using L = MergeWarp<V, NUMERIC>;
     constexpr bool HV = NUMERIC && VOps<V>::has_val;
-    constexpr int NWORDS = W / 32;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr long long kFar = 0x7fffffffffffffffLL;
+    V* acc = reinterpret_cast<V*>(smem);
+    unsigned* bits = reinterpret_cast<unsigned*>(smem + L::kBitsAt);
+    unsigned short* before = reinterpret_cast<unsigned short*>(smem + L::kBeforeAt);
+    unsigned short* list = reinterpret_cast<unsigned short*>(smem + L::kListAt);
+    unsigned short* outs = reinterpret_cast<unsigned short*>(smem + L::kOutAt);
     const int lane = lane_id();
-    const int w = threadIdx.x >> 5;
-    constexpr size_t vbytes = HV ? sizeof(V) * W : 0;
-    unsigned char* base = smem_raw + (size_t)w * (vbytes + W / 8);
-    V* acc = reinterpret_cast<V*>(base);
-    unsigned* bm = reinterpret_cast<unsigned*>(base + vbytes);
-    for (int s = lane; s < W; s += 32)
-        if constexpr (HV) acc[s] = VOps<V>::init();
-    for (int t = lane; t < NWORDS; t += 32) bm[t] = 0u;
+    const IT* mycol = lane < c ? parts.col[lane] : nullptr;
+    long long count = 0;
+    // each list's share of the next chunk, its first column and the column
+    // after its share: loaded as soon as the chunk before has taken its part
+    long long total = 0, share = 0, head = kFar, next = kFar;
+    auto offer = [&]() {
+        const long long left = end - cur;
+        total = warp_sum(left);
+        share = left;
+        if (total > L::kS) share = min(left, (long long)(L::kS - 8 * c) * left / total + 8);
+        head = left > 0 ? (long long)mycol[cur] : kFar;
+        next = share < left ? (long long)mycol[cur + share] : kFar;
+    };
+    offer();
+    while (total > 0) {
+        const long long c0 = warp_min(head);
+        const long long c1 = min(warp_min(next), c0 + kMergeSpan);
+        // columns: bits of the map, offsets in list order; four lists' loads
+        // are in flight together
+        int mine = 0;     // entries of list `lane` in the chunk
+        int base = 0;
+        int top = 0;      // one past the largest offset
+        for (int s0 = 0; s0 < c; s0 += 4) {
+            const IT* col[4];
+            int lim[4];
+            IT j[4][4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int s = min(s0 + u, c - 1);
+                lim[u] = s0 + u < c ? __shfl_sync(kFull, (int)share, s) : 0;
+                col[u] = parts.col[s] + __shfl_sync(kFull, cur, s);
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    j[u][t] = 32 * t + lane < lim[u] ? col[u][32 * t + lane] : IT(0);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                int n = 0;
+                for (int x0 = 0; x0 < lim[u]; x0 += 128) {
+                    if (x0 > 0) {
+#pragma unroll
+                        for (int t = 0; t < 4; ++t)
+                            j[u][t] = x0 + 32 * t + lane < lim[u] ? col[u][x0 + 32 * t + lane] : IT(0);
+                    }
+                    int got = 0;
+#pragma unroll
+                    for (int t = 0; t < 4; ++t) {
+                        const bool in =
+                            x0 + 32 * t + lane < lim[u] && (long long)j[u][t] < c1;
+                        if (in) {
+                            const int d = (int)((long long)j[u][t] - c0);
+                            atomicOr(&bits[d >> 5], 1u << (d & 31));
+                            if constexpr (HV) list[base + x0 + 32 * t + lane] = (unsigned short)d;
+                            top = max(top, d + 1);
+                        }
+                        got += __popc(__ballot_sync(kFull, in));
+                    }
+                    n += got;
+                    if (got < 128) break;
+                }
+                mine = lane == s0 + u ? n : mine;
+                base += n;
+            }
+        }
+        const long long from = cur;   // where the chunk's part of list `lane` begins
+        cur += mine;
+        offer();
+        const int nwords = ((int)__reduce_max_sync(kFull, (unsigned)top) + 31) >> 5;
+        __syncwarp();
+        if constexpr (!NUMERIC) {
+            for (int t = lane; t < nwords; t += 32) {
+                count += __popc(bits[t]);
+                bits[t] = 0u;
+            }
+            __syncwarp();
+            continue;
+        }
+        // outputs before each word; without values the columns are written here
+        int n_out = 0;
+        for (int w0 = 0; w0 < nwords; w0 += 128) {
+            uint4 x = *reinterpret_cast<const uint4*>(bits + w0 + 4 * lane);
+            const int p0 = __popc(x.x), p1 = p0 + __popc(x.y), p2 = p1 + __popc(x.z),
+                      p3 = p2 + __popc(x.w);
+            const int incl = warp_incl_scan(p3);
+            const int b = n_out + incl - p3;
+            ushort4 y;
+            y.x = (unsigned short)b;
+            y.y = (unsigned short)(b + p0);
+            y.z = (unsigned short)(b + p1);
+            y.w = (unsigned short)(b + p2);
+            *reinterpret_cast<ushort4*>(before + w0 + 4 * lane) = y;
+            n_out += __shfl_sync(kFull, incl, 31);
+        }
+        __syncwarp();
+        if constexpr (HV) {
+            base = 0;
+            for (int s0 = 0; s0 < c; s0 += 4) {
+                const V* val[4];
+                int n[4];
+                V v[4][4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const int s = min(s0 + u, c - 1);
+                    n[u] = s0 + u < c ? __shfl_sync(kFull, mine, s) : 0;
+                    val[u] = parts.val[s] + __shfl_sync(kFull, from, s);
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+                        if (32 * t + lane < n[u]) v[u][t] = val[u][32 * t + lane];
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    for (int x0 = 0; x0 < n[u]; x0 += 128) {
+                        if (x0 > 0) {
+#pragma unroll
+                            for (int t = 0; t < 4; ++t)
+                                if (x0 + 32 * t + lane < n[u]) v[u][t] = val[u][x0 + 32 * t + lane];
+                        }
+#pragma unroll
+                        for (int t = 0; t < 4; ++t) {
+                            const int x = x0 + 32 * t + lane;
+                            if (x < n[u]) {
+                                const int d = list[base + x];
+                                const int slot = before[d >> 5] +
+                                                 __popc(bits[d >> 5] & ~(0xffffffffu << (d & 31)));
+                                if (kStoreFirst<V> && s0 + u == 0) acc[slot] = v[u][t];
+                                else acc[slot] = VOps<V>::add(acc[slot], v[u][t]);
+                                outs[slot] = (unsigned short)d;
+                            }
+                        }
+                    }
+                    base += n[u];
+                    __syncwarp();
+                }
+            }
+        } else {
+            // the places of the columns from the bits alone
+            for (int t = lane; t < nwords; t += 32) {
+                int p = before[t];
+                for (unsigned word = bits[t]; word; word &= word - 1u)
+                    outs[p++] = (unsigned short)(32 * t + __ffs(word) - 1);
+            }
+            __syncwarp();
+        }
+        for (int t = lane; t < n_out; t += 32) {
+            const long long pos = out + count + t;
+            if (pos < out_end) {
+                ciC[pos] = (IT)(c0 + outs[t]);
+                if constexpr (HV) vC[pos] = acc[t];
+            }
+            if constexpr (HV) acc[t] = VOps<V>::init();
+        }
+        for (int t = lane; t < nwords; t += 32) bits[t] = 0u;
+        __syncwarp();
+        count += n_out;
+    }
+    if constexpr (!NUMERIC) count = warp_sum(count);
+    return count;
+}
+
+template <class IT, class V, bool NUMERIC>
+__device__ __forceinline__ unsigned char* merge_warp_memory(unsigned char* smem_raw) {
+    using L = MergeWarp<V, NUMERIC>;
+    unsigned char* smem = smem_raw + (size_t)(threadIdx.x >> 5) * L::kBytes;
+    if constexpr (NUMERIC && VOps<V>::has_val) {
+        V* acc = reinterpret_cast<V*>(smem);
+        for (int t = lane_id(); t < L::kS; t += 32) acc[t] = VOps<V>::init();
+    }
+    unsigned* bits = reinterpret_cast<unsigned*>(smem + L::kBitsAt);
+    for (int t = lane_id(); t < L::kWords; t += 32) bits[t] = 0u;
     __syncwarp();
-    // rows are taken one at a time from a counter: row sizes are heavy-tailed,
-    // so a fixed stride would leave some warps with far more work
+    return smem;
+}
+
+// Rows, one at a time per warp from a counter (row sizes are heavy-tailed).
+// Rows of more than kMergeLong entries are put on `longs` (if given) while it
+// has room, and left to the segment kernels.
+template <class IT, class V, bool NUMERIC>
+__global__ void __launch_bounds__(kMergeWarps * 32)
+    merge_rows_kernel(int c, MergeParts<IT, V> parts, long long m, int64_t* __restrict__ rowcnt,
+                      const int64_t* __restrict__ rpC, IT* __restrict__ ciC, V* __restrict__ vC,
+                      int* err, unsigned long long* work, MergeLong* longs) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned char* smem = merge_warp_memory<IT, V, NUMERIC>(smem_raw);
+    const int lane = lane_id();
     while (true) {
         long long i = 0;
         if (lane == 0) i = (long long)atomicAdd(work, 1ull);
         i = __shfl_sync(kFull, i, 0);
         if (i >= m) break;
-        long long b_own = 0, e_own = 0;
+        long long cur = 0, end = 0;
         if (lane < c) {
-            b_own = parts.rp[lane][i];
-            e_own = parts.re[lane] ? parts.re[lane][i] : parts.rp[lane][i + 1];
+            cur = parts.rp[lane][i];
+            end = parts.re[lane] ? parts.re[lane][i] : parts.rp[lane][i + 1];
         }
-        long long wb[CM];  // position of window A's first entry (warp-uniform)
-        long long we[CM];  // end of list s in row i
-        int off[CM];       // entries of window A already consumed
-        IT ja[CM], jb[CM], jc[CM];
-        V va[CM], vb[CM], vc[CM];
-#pragma unroll
-        for (int s = 0; s < CM; ++s) {
-            wb[s] = __shfl_sync(kFull, b_own, s);
-            we[s] = s < c ? __shfl_sync(kFull, e_own, s) : 0;
-            off[s] = 0;
-            const long long qa = wb[s] + lane, qb = qa + 32, qc = qa + 64;
-            ja[s] = qa < we[s] ? parts.col[s][qa] : IT(0);
-            jb[s] = qb < we[s] ? parts.col[s][qb] : IT(0);
-            jc[s] = qc < we[s] ? parts.col[s][qc] : IT(0);
-            va[s] = V{};
-            vb[s] = V{};
-            vc[s] = V{};
-            if constexpr (HV) {
-                if (qa < we[s]) va[s] = parts.val[s][qa];
-                if (qb < we[s]) vb[s] = parts.val[s][qb];
-                if (qc < we[s]) vc[s] = parts.val[s][qc];
-            }
-        }
-        long long out = NUMERIC ? rpC[i] : 0;
-        const long long out_end = NUMERIC ? rpC[i + 1] : 0;
-        long long count = 0;
-        while (true) {
-            long long nxt = n;
-#pragma unroll
-            for (int s = 0; s < CM; ++s) {
-                const long long h = (long long)__shfl_sync(kFull, ja[s], off[s] & 31);
-                if (wb[s] + off[s] < we[s]) nxt = min(nxt, h);
-            }
-            if (nxt >= n) break;
-            const long long c0 = (nxt / W) * W;
-            const long long c1 = min(c0 + (long long)W, n);
-#pragma unroll
-            for (int s = 0; s < CM; ++s) {
-                while (true) {
-                    const bool valid =
-                        lane >= off[s] && wb[s] + lane < we[s] && (long long)ja[s] < c1;
-                    const int slot = (int)((long long)ja[s] - c0);
-                    if (valid) {
-                        atomicOr(&bm[slot >> 5], 1u << (slot & 31));
-                        if constexpr (HV) {
-                            if (kStoreFirst<V> && s == 0) acc[slot] = va[s];
-                            else acc[slot] = VOps<V>::add(acc[slot], va[s]);
-                        }
-                    }
-                    __syncwarp();
-                    off[s] += __popc(__ballot_sync(kFull, valid));
-                    if (off[s] < 32) break;
-                    // window A used up: B and C move up, the window after C is loaded
-                    wb[s] += 32;
-                    off[s] = 0;
-                    ja[s] = jb[s];
-                    va[s] = vb[s];
-                    jb[s] = jc[s];
-                    vb[s] = vc[s];
-                    const long long qc = wb[s] + 64 + lane;
-                    if (qc < we[s]) {
-                        jc[s] = parts.col[s][qc];
-                        if constexpr (HV) vc[s] = parts.val[s][qc];
-                    }
-                    if (wb[s] >= we[s]) break;
+        if (longs && warp_sum(end - cur) > kMergeLong) {
+            unsigned at = 0;
+            if (lane == 0) at = atomicAdd(&longs->count, 1u);
+            at = __shfl_sync(kFull, at, 0);
+            if (at < kMergeLongRows) {
+                if (lane == 0) {
+                    longs->row[at] = i;
+                    if constexpr (!NUMERIC) rowcnt[i] = 0;
                 }
+                continue;
             }
-            // emit the chunk (numeric) or add up its columns (count), clearing it
+        }
+        const long long out = NUMERIC ? rpC[i] : 0, out_end = NUMERIC ? rpC[i + 1] : 0;
+        const long long got =
+            merge_range<IT, V, NUMERIC>(c, parts, cur, end, out, out_end, ciC, vC, smem);
+        if (lane == 0) {
+            if constexpr (!NUMERIC) rowcnt[i] = got;
+            else if (out + got != out_end) atomicExch(err, (int)kDevCountMismatch);
+        }
+    }
+}
+
+// The listed rows: a warp takes one column segment of one row.  NUMERIC:
+// places follow from the counts of the row's earlier segments; else the
+// segment's outputs are counted (and added to the row's count, if wanted).
+template <class IT, class V, bool NUMERIC>
+__global__ void __launch_bounds__(kMergeWarps * 32)
+    merge_segments_kernel(int c, MergeParts<IT, V> parts, int64_t* __restrict__ rowcnt, const int64_t* __restrict__ rpC,
+                          IT* __restrict__ ciC, V* __restrict__ vC, int* err,
+                          unsigned long long* work, MergeLong* longs) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned char* smem = merge_warp_memory<IT, V, NUMERIC>(smem_raw);
+    const int lane = lane_id();
+    const long long units = (long long)min(longs->count, (unsigned)kMergeLongRows) * kMergeSegs;
+    while (true) {
+        long long u = 0;
+        if (lane == 0) u = (long long)atomicAdd(work, 1ull);
+        u = __shfl_sync(kFull, u, 0);
+        if (u >= units) break;
+        const int g = (int)(u % kMergeSegs);
+        const long long i = longs->row[u / kMergeSegs];
+        long long cur = 0, end = 0, lo = 0x7fffffffffffffffLL, hi = 0;
+        const IT* col = nullptr;
+        if (lane < c) {
+            col = parts.col[lane];
+            cur = parts.rp[lane][i];
+            end = parts.re[lane] ? parts.re[lane][i] : parts.rp[lane][i + 1];
+            if (cur < end) {
+                lo = (long long)col[cur];
+                hi = (long long)col[end - 1] + 1;
+            }
+        }
+        // the row's columns [lo, hi) cut into equal segments
+        lo = warp_min(lo);
+        hi = warp_max(hi);
+        const long long per = (hi - lo) / kMergeSegs, rest = (hi - lo) % kMergeSegs;
+        auto bound = [&](int t) { return lo + per * t + rest * t / kMergeSegs; };
+        auto first_from = [&](long long p, long long e, long long key) {
+            while (p < e) {
+                const long long mid = (p + e) >> 1;
+                if ((long long)col[mid] < key) p = mid + 1;
+                else e = mid;
+            }
+            return p;
+        };
+        if (g > 0) cur = first_from(cur, end, bound(g));
+        if (g + 1 < kMergeSegs) end = first_from(cur, end, bound(g + 1));
+        __syncwarp();
+        long long out = 0, out_end = 0;
+        if constexpr (NUMERIC) {
+            const long long k = lane < kMergeSegs ? longs->seg[u / kMergeSegs * kMergeSegs + lane] : 0;
+            out = rpC[i] + warp_sum(lane < g ? k : 0);
+            out_end = min(out + __shfl_sync(kFull, k, g), (long long)rpC[i + 1]);
+        }
+        const long long got =
+            merge_range<IT, V, NUMERIC>(c, parts, cur, end, out, out_end, ciC, vC, smem);
+        if (lane == 0) {
             if constexpr (NUMERIC) {
-                for (int t0 = 0; t0 < NWORDS; t0 += 32) {
-                    const int t = t0 + lane;
-                    unsigned word = t < NWORDS ? bm[t] : 0u;
-                    const int pc = __popc(word);
-                    const int incl = warp_incl_scan(pc);
-                    long long pos = out + incl - pc;
-                    while (word) {
-                        const int b = __ffs(word) - 1;
-                        word &= word - 1;
-                        const int slot = t * 32 + b;
-                        if (pos < out_end) {
-                            ciC[pos] = (IT)(c0 + slot);
-                            if constexpr (HV) vC[pos] = acc[slot];
-                        }
-                        if constexpr (HV) acc[slot] = VOps<V>::init();
-                        ++pos;
-                    }
-                    if (t < NWORDS) bm[t] = 0u;
-                    out += __shfl_sync(kFull, incl, 31);
-                }
+                if (out + got != out_end || (g + 1 == kMergeSegs && out_end != rpC[i + 1]))
+                    atomicExch(err, (int)kDevCountMismatch);
             } else {
-                // only the row total is needed: per-lane counts, summed once
-                for (int t = lane; t < NWORDS; t += 32) {
-                    count += __popc(bm[t]);
-                    bm[t] = 0u;
-                }
+                longs->seg[u] = got;
+                if (rowcnt) atomicAdd((unsigned long long*)&rowcnt[i], (unsigned long long)got);
             }
-            __syncwarp();
-        }
-        if constexpr (!NUMERIC) {
-            count = warp_sum(count);
-            if (lane == 0) rowcnt[i] = count;
-        } else {
-            if (lane == 0 && out != out_end) atomicExch(err, (int)kDevCountMismatch);
         }
     }
 }
@@ -285,8 +378,8 @@ __global__ void __launch_bounds__(WARPS * 32)
 // records kDevWaitTimeout, lets the copies it issued land, and ends the
 // warp's work).  Windows start at multiples of four entries (16 bytes of
 // int32 columns, 32 of float64 values); the last entries of an array that a
-// 16-byte copy cannot reach are loaded by the lanes.  Entries are then
-// consumed in column order chunk by chunk exactly as in merge_win_kernel.
+// 16-byte copy cannot reach are loaded by the lanes.  Entries are
+// then consumed in column order, chunk by chunk of W columns.
 __device__ __forceinline__ unsigned smem_u32(const void* p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
@@ -532,145 +625,53 @@ __global__ void __launch_bounds__(WARPS * 32)
     }
 }
 
-// The count of the merge for int32 columns in 16-byte aligned arrays: the
-// same sweep with four columns per lane per load (128 entries per window),
-// so four times the bytes of every list are in flight.  Entry x of a window
-// is component x % 4 of lane x / 4; windows start at multiples of four
-// entries, and entries outside [row begin, row end) are masked by position.
-__device__ __forceinline__ int4 merge_load4(const int32_t* __restrict__ col, long long q,
-                                            long long len) {
-    if (q + 4 <= len) return *reinterpret_cast<const int4*>(col + q);
-    int4 r = make_int4(0, 0, 0, 0);
-    if (q < len) r.x = col[q];
-    if (q + 1 < len) r.y = col[q + 1];
-    if (q + 2 < len) r.z = col[q + 2];
-    if (q + 3 < len) r.w = col[q + 3];
-    return r;
-}
-
-__device__ __forceinline__ int comp4(const int4& v, int j) {
-    return j == 0 ? v.x : j == 1 ? v.y : j == 2 ? v.z : v.w;
-}
-
-template <class V, int W, int WARPS, int CM>
-__global__ void __launch_bounds__(WARPS * 32)
-    merge_count4_kernel(int c, MergeParts<int32_t, V> parts, long long m, long long n,
-                        int64_t* __restrict__ rowcnt, unsigned long long* work) {
-    constexpr int NWORDS = W / 32;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int lane = lane_id();
-    const int w = threadIdx.x >> 5;
-    unsigned* bm = reinterpret_cast<unsigned*>(smem_raw + (size_t)w * (W / 8));
-    for (int t = lane; t < NWORDS; t += 32) bm[t] = 0u;
-    __syncwarp();
-    while (true) {
-        long long i = 0;
-        if (lane == 0) i = (long long)atomicAdd(work, 1ull);
-        i = __shfl_sync(kFull, i, 0);
-        if (i >= m) break;
-        long long b_own = 0, e_own = 0;
-        if (lane < c) {
-            b_own = parts.rp[lane][i];
-            e_own = parts.re[lane] ? parts.re[lane][i] : parts.rp[lane][i + 1];
-        }
-        long long wb[CM], we[CM];
-        int off[CM];
-        int4 xa[CM], xb[CM], xc[CM];
-#pragma unroll
-        for (int s = 0; s < CM; ++s) {
-            const long long b = __shfl_sync(kFull, b_own, s);
-            we[s] = s < c ? __shfl_sync(kFull, e_own, s) : 0;
-            wb[s] = b & ~3LL;
-            off[s] = (int)(b - wb[s]);
-            xa[s] = xb[s] = xc[s] = make_int4(0, 0, 0, 0);
-            if (b < we[s]) {
-                const long long q = wb[s] + 4 * lane;
-                xa[s] = merge_load4(parts.col[s], q, parts.len[s]);
-                if (wb[s] + 128 < we[s]) xb[s] = merge_load4(parts.col[s], q + 128, parts.len[s]);
-                if (wb[s] + 256 < we[s]) xc[s] = merge_load4(parts.col[s], q + 256, parts.len[s]);
-            }
-        }
-        long long count = 0;
-        while (true) {
-            long long nxt = n;
-#pragma unroll
-            for (int s = 0; s < CM; ++s) {
-                const int h = __shfl_sync(kFull, comp4(xa[s], off[s] & 3), (off[s] >> 2) & 31);
-                if (wb[s] + off[s] < we[s]) nxt = min(nxt, (long long)h);
-            }
-            if (nxt >= n) break;
-            const long long c0 = (nxt / W) * W;
-            const long long c1 = min(c0 + (long long)W, n);
-#pragma unroll
-            for (int s = 0; s < CM; ++s) {
-                while (true) {
-                    int got = 0;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int e = 4 * lane + j;
-                        const long long col = comp4(xa[s], j);
-                        const bool valid = e >= off[s] && wb[s] + e < we[s] && col < c1;
-                        if (valid) {
-                            const int slot = (int)(col - c0);
-                            atomicOr(&bm[slot >> 5], 1u << (slot & 31));
-                        }
-                        got += __popc(__ballot_sync(kFull, valid));
-                    }
-                    off[s] += got;
-                    if (off[s] < 128) break;
-                    // window A used up: B and C move up, the window after C is loaded
-                    wb[s] += 128;
-                    off[s] = 0;
-                    xa[s] = xb[s];
-                    xb[s] = xc[s];
-                    if (wb[s] + 256 < we[s])
-                        xc[s] = merge_load4(parts.col[s], wb[s] + 256 + 4 * lane, parts.len[s]);
-                    if (wb[s] >= we[s]) break;
-                }
-            }
-            __syncwarp();
-            for (int t = lane; t < NWORDS; t += 32) {
-                count += __popc(bm[t]);
-                bm[t] = 0u;
-            }
-            __syncwarp();
-        }
-        count = warp_sum(count);
-        if (lane == 0) rowcnt[i] = count;
+template <class IT, class V, bool NUMERIC, class K>
+cudaError_t merge_grid(K k, long long units, int sm_count, size_t* smem, unsigned* grid) {
+    *smem = (size_t)kMergeWarps * MergeWarp<V, NUMERIC>::kBytes;
+    if (*smem > 48 * 1024) {
+        cudaError_t e =
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)*smem);
+        if (e != cudaSuccess) return e;
     }
+    int occ = 1;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kMergeWarps * 32, *smem);
+    if (occ < 1) occ = 1;
+    *grid = (unsigned)std::max<long long>(
+        1, std::min((units + kMergeWarps - 1) / kMergeWarps, (long long)sm_count * occ));
+    return cudaSuccess;
+}
+
+template <class IT, class V, bool NUMERIC>
+cudaError_t launch_merge_segments(int c, const MergeParts<IT, V>& mp, int sm_count,
+                                  cudaStream_t s, int64_t* rowcnt, const int64_t* rpC, IT* colC,
+                                  V* valC, int* err, MergeLong* longs) {
+    auto k = merge_segments_kernel<IT, V, NUMERIC>;
+    size_t smem = 0;
+    unsigned g = 1;
+    cudaError_t e = merge_grid<IT, V, NUMERIC>(k, (long long)kMergeLongRows * kMergeSegs, sm_count,
+                                               &smem, &g);
+    if (e != cudaSuccess) return e;
+    count_launches(1);
+    k<<<g, kMergeWarps * 32, smem, s>>>(c, mp, rowcnt, rpC, colC, valC, err,
+                                        &longs->work[NUMERIC ? 1 : 0], longs);
+    return cudaGetLastError();
 }
 
 template <class IT, class V, bool NUMERIC>
 cudaError_t launch_merge_t(int c, const spgemm_csr* parts, long long m, long long n,
                            int sm_count, cudaStream_t s, int64_t* rowcnt, const int64_t* rpC,
                            void* colC, void* valC, int* err, unsigned long long* work,
-                           bool staged_opt) {
+                           MergeLong* longs, bool staged_opt) {
+    if (m <= 0) return cudaSuccess;
     MergeParts<IT, V> mp{};
-    bool aligned16 = true;
+    long long entries = 0;   // at most: a part's arrays may hold more than its rows
     for (int t = 0; t < c; ++t) {
         mp.rp[t] = parts[t].rowptr;
         mp.re[t] = parts[t].rowend;
         mp.col[t] = (const IT*)parts[t].col;
         mp.val[t] = (const V*)parts[t].val;
         mp.len[t] = parts[t].nnz;
-        aligned16 = aligned16 && ((uintptr_t)parts[t].col % 16) == 0;
-    }
-    if constexpr (!NUMERIC && std::is_same<IT, int32_t>::value) {
-        if (c <= 4 && aligned16) {
-            constexpr int W = 8192, WARPS = 4;
-            auto k = c <= 2 ? merge_count4_kernel<V, W, WARPS, 2> : merge_count4_kernel<V, W, WARPS, 4>;
-            const size_t smem = (size_t)WARPS * (W / 8);
-            int occ = 1;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, WARPS * 32, smem);
-            if (occ < 1) occ = 1;
-            const long long need = (m + WARPS - 1) / WARPS;
-            const long long g = std::max<long long>(1, std::min(need, (long long)sm_count * occ));
-            if (m > 0) {
-                count_launches(1);
-                k<<<(unsigned)g, WARPS * 32, smem, s>>>(c, mp, m, n, rowcnt, work);
-            }
-            return cudaGetLastError();
-        }
+        entries += parts[t].nnz;
     }
     if constexpr (NUMERIC) {
         bool staged = staged_opt && c <= 4;
@@ -693,75 +694,47 @@ cudaError_t launch_merge_t(int c, const spgemm_csr* parts, long long m, long lon
             if (occ < 1) occ = 1;
             const long long need = (m + WARPS - 1) / WARPS;
             const long long g = std::max<long long>(1, std::min(need, (long long)sm_count * occ));
-            if (m > 0) {
-                count_launches(1);
-                k<<<(unsigned)g, WARPS * 32, smem, s>>>(c, mp, m, n, rpC, (IT*)colC, (V*)valC,
-                                                        err, work);
-            }
+            count_launches(1);
+            k<<<(unsigned)g, WARPS * 32, smem, s>>>(c, mp, m, n, rpC, (IT*)colC, (V*)valC, err, work);
             return cudaGetLastError();
         }
     }
-    if (c <= 8) {
-        // the count keeps only a bitmap, so its chunks can be wider
-        constexpr int W = NUMERIC ? 1024 : 8192, WARPS = 8;
-        auto k = c <= 2   ? merge_win_kernel<IT, V, W, WARPS, NUMERIC, 2>
-                 : c <= 4 ? merge_win_kernel<IT, V, W, WARPS, NUMERIC, 4>
-                          : merge_win_kernel<IT, V, W, WARPS, NUMERIC, 8>;
-        constexpr size_t vb = (NUMERIC && VOps<V>::has_val) ? sizeof(V) : 0;
-        const size_t smem = (size_t)WARPS * (W * vb + W / 8);
-        if (smem > 48 * 1024) {
-            cudaError_t e =
-                cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        int occ = 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, WARPS * 32, smem);
-        if (occ < 1) occ = 1;
-        const long long need = (m + WARPS - 1) / WARPS;
-        const long long g = std::max<long long>(1, std::min(need, (long long)sm_count * occ));
-        if (m > 0) {
-            count_launches(1);
-            k<<<(unsigned)g, WARPS * 32, smem, s>>>(c, mp, m, n, rowcnt, rpC, (IT*)colC,
-                                                    (V*)valC, err, work);
-        }
-        return cudaGetLastError();
-    }
-    constexpr int W = 2048, WARPS = 4;
-    auto k = merge_kernel<IT, V, W, WARPS, NUMERIC>;
-    constexpr size_t vb = (NUMERIC && VOps<V>::has_val) ? sizeof(V) : 0;
-    size_t smem = (size_t)WARPS * (W * vb + W / 8);
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
-    int occ = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, WARPS * 32, smem);
-    if (occ < 1) occ = 1;
-    long long need = (m + WARPS - 1) / WARPS;
-    long long g = std::max<long long>(1, std::min(need, (long long)sm_count * occ));
-    if (m > 0) {
-        count_launches(1);
-        k<<<(unsigned)g, WARPS * 32, smem, s>>>(c, mp, m, n, rowcnt, rpC, (IT*)colC, (V*)valC, err);
-    }
-    return cudaGetLastError();
+    if (entries <= kMergeLong) longs = nullptr;   // no row can be long
+    cudaError_t e;
+    if (longs && (e = cudaMemsetAsync(longs, 0, kMergeLongHead, s)) != cudaSuccess) return e;
+    auto k = merge_rows_kernel<IT, V, NUMERIC>;
+    size_t smem = 0;
+    unsigned g = 1;
+    if ((e = merge_grid<IT, V, NUMERIC>(k, m, sm_count, &smem, &g)) != cudaSuccess) return e;
+    count_launches(1);
+    k<<<g, kMergeWarps * 32, smem, s>>>(c, mp, m, rowcnt, rpC, (IT*)colC, (V*)valC, err, work, longs);
+    if ((e = cudaGetLastError()) != cudaSuccess || !longs) return e;
+    // the listed rows' segments: counted, and for the numeric pass then filled
+    e = launch_merge_segments<IT, V, false>(c, mp, sm_count, s, NUMERIC ? nullptr : rowcnt,
+                                            nullptr, nullptr, nullptr, err, longs);
+    if constexpr (NUMERIC)
+        if (e == cudaSuccess)
+            e = launch_merge_segments<IT, V, true>(c, mp, sm_count, s, nullptr, rpC, (IT*)colC,
+                                                   (V*)valC, err, longs);
+    return e;
 }
 
 cudaError_t launch_merge(int c, const spgemm_csr* parts, int vt, long long m, long long n,
                          int sm_count, cudaStream_t s, bool numeric, int64_t* rowcnt,
                          const int64_t* rpC, void* colC, void* valC, int* err,
-                         unsigned long long* work, bool staged) {
+                         unsigned long long* work, MergeLong* longs, bool staged) {
     const bool i32 = parts[0].index_type == SPGEMM_INDEX_I32;
     return with_value_type(vt, [&](auto tag) -> cudaError_t {
         using V = decltype(tag);
         if (numeric)
             return i32 ? launch_merge_t<int32_t, V, true>(c, parts, m, n, sm_count, s, rowcnt, rpC,
-                                                          colC, valC, err, work, staged)
+                                                          colC, valC, err, work, longs, staged)
                        : launch_merge_t<int64_t, V, true>(c, parts, m, n, sm_count, s, rowcnt, rpC,
-                                                          colC, valC, err, work, staged);
+                                                          colC, valC, err, work, longs, staged);
         return i32 ? launch_merge_t<int32_t, V, false>(c, parts, m, n, sm_count, s, rowcnt, rpC,
-                                                       colC, valC, err, work, staged)
+                                                       colC, valC, err, work, longs, staged)
                    : launch_merge_t<int64_t, V, false>(c, parts, m, n, sm_count, s, rowcnt, rpC,
-                                                       colC, valC, err, work, staged);
+                                                       colC, valC, err, work, longs, staged);
     });
 }
 

@@ -126,7 +126,7 @@ spgemm_status spgemm_merge_symbolic_static(int32_t c, const spgemm_csr* parts,
         (e = cudaMemsetAsync(rowptrC + m, 0, sizeof(int64_t), s)) != cudaSuccess)
         return static_fail(SPGEMM_ERR_CUDA, cudaGetErrorString(e));
     e = sg::launch_merge(c, parts, vt, m, n, sms, s, false, rowptrC, nullptr, nullptr, nullptr,
-                         &cnt->err, &cnt->work_counter[0]);
+                         &cnt->err, &cnt->work_counter[0], nullptr);
     if (e == cudaSuccess) e = sg::launch_exclusive_scan(rowptrC, m + 1, partials, s);
     int64_t total = 0;
     int herr = 0;

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cstddef>
 #include <cstdint>
 #include <string>
 #include <vector>
@@ -137,10 +138,26 @@ template <class IT, class V>
 cudaError_t launch_numeric(Plan& P, unsigned char* ws, const int64_t* rpC, long long cap,
                            void* colC, void* valC, int64_t* rowend = nullptr,
                            int32_t* overflow = nullptr, unsigned* overflow_count = nullptr);
+// Rows of a merge with more than kMergeLong entries over all lists, each cut
+// into kMergeSegs column segments (scratch of one merge call).
+constexpr int kMergeLongRows = 4096;
+constexpr int kMergeSegs = 16;
+constexpr long long kMergeLong = 8192;
+constexpr size_t kMergeLongHead = 64;   // the bytes a call clears first
+struct MergeLong {
+    unsigned count;                     // rows found (those past kMergeLongRows are merged whole)
+    unsigned pad;
+    unsigned long long work[2];         // segments handed out: count, fill
+    unsigned long long pad2[5];
+    long long row[kMergeLongRows];
+    long long seg[kMergeLongRows * kMergeSegs];   // outputs of every segment
+};
+static_assert(offsetof(MergeLong, row) == kMergeLongHead, "the head is cleared, not the lists");
 cudaError_t launch_merge(int c, const spgemm_csr* parts, int vt, long long m, long long n,
                          int sm_count, cudaStream_t s, bool numeric, int64_t* rowcnt,
                          const int64_t* rpC, void* colC, void* valC, int* err,
                          unsigned long long* work,   // work: zeroed row counter
+                         MergeLong* longs,           // scratch for long rows, or NULL
                          bool staged = false);       // numeric: stage lists by bulk copies
 template <class IT>
 cudaError_t launch_kslice_bounds(const spgemm_csr& A, int c, int64_t* bounds, int sm_count,

@@ -389,3 +389,60 @@ def test_short_rows_over_many_a_entries(sg, idt):
     assert np.array_equal(Lc.rowptr.cpu().numpy(), R.rowptr)
     assert np.array_equal(Lc.col.cpu().numpy().astype(np.int64), R.col)
     assert np.array_equal(Lc.val.cpu().numpy(), R.val)
+
+
+@pytest.mark.parametrize("c", [1, 2, 4, 9, 32])
+@pytest.mark.parametrize("value", ["u01_f64", "u11_f32", "int", "none"])
+def test_merge_row_sizes(sg, c, value):
+    """Row totals at the edges of a numeric chunk (512 entries), a count chunk
+    (2048) and of the rows cut into segments (beyond 8192); columns that fill a
+    chunk's span (16384), that leave gaps wider than it, and lists of very
+    unequal length."""
+    rng = np.random.default_rng(c)
+    totals = [0, 1, 2, 31, 511, 512, 513, 2047, 2048, 2049, 8191, 8192, 8193, 20000]
+    n = 200_000
+    rows = [(t, span, skew) for t in totals for span in (0, 16384, n) for skew in (False, True)]
+    parts = []
+    for s in range(c):
+        cols = []
+        for t, span, skew in rows:
+            k = t // c if not skew else (t - (c - 1) * (t // (8 * c)) if s == 0 else t // (8 * c))
+            width = max(k, span if span else t)        # span 0: columns side by side
+            pick = rng.choice(width, size=k, replace=False) if width else np.zeros(0, np.int64)
+            cols.append(np.sort(pick) + (n - width if skew else 0))
+        lens = [x.size for x in cols]
+        col = np.concatenate(cols)
+        rp = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+        parts.append(inputs.CSR(len(rows), n, rp, col.astype(np.int32 if c % 2 else np.int64),
+                                inputs.draw_values(rng, col.size, value)))
+    sr = 1 if value == "none" else 0
+    C = sg.merge([sg.to_device(P) for P in parts], semiring=sr, verify=True)
+    S = oracle.sum_partials([oracle.OCSR(P.nrows, P.ncols, P.rowptr, P.col.astype(np.int64),
+                                         None if P.val is None else P.val.astype(
+                                             np.float64 if value == "u11_f32" else P.val.dtype))
+                             for P in parts])
+    rp, col, val = C.to_host()
+    assert np.array_equal(rp, S.rowptr) and np.array_equal(col.astype(np.int64), S.col)
+    if value == "u11_f32":
+        # c - 1 additions of float32, each rounded to at most u = 2^-24 of a sum below c
+        assert np.all(np.abs(val - S.val) <= (c - 1) * c * 2.0 ** -24)
+    elif val is not None:
+        assert np.array_equal(val, S.val)
+
+
+def test_merge_more_long_rows_than_listed(sg):
+    """More rows of over 8192 entries than the list of long rows holds (4096):
+    the others are merged whole.  Even and odd columns give every column."""
+    import torch
+
+    m, n = 4200, 8400
+    cols = torch.arange(n, device="cuda", dtype=torch.int32)
+    parts = []
+    for s in (0, 1):
+        rp = torch.arange(m + 1, device="cuda", dtype=torch.int64) * (n // 2)
+        col = cols[s::2].repeat(m)
+        parts.append(sg.DeviceCSR(m, n, rp, col, col.double()))
+    C = sg.merge(parts, verify=True)
+    assert bool((C.rowptr == torch.arange(m + 1, device="cuda") * n).all())
+    assert bool((C.col.view(m, n) == cols).all())
+    assert bool((C.val.view(m, n) == cols.double()).all())
