@@ -446,3 +446,42 @@ def test_merge_more_long_rows_than_listed(sg):
     assert bool((C.rowptr == torch.arange(m + 1, device="cuda") * n).all())
     assert bool((C.col.view(m, n) == cols).all())
     assert bool((C.val.view(m, n) == cols.double()).all())
+
+
+@pytest.mark.parametrize("n", [900, (1 << 25) - 1, 1 << 25])
+@pytest.mark.parametrize("value", ["u01_f64", "int", "none"])
+def test_rows_of_33_to_128_products(sg, n, value):
+    """Rows around the bounds of the register sort (64 and 128 products) with
+    all columns distinct, all equal and mixed, over many A entries and over
+    few, the last column among them; n = 2^25 is the first width whose rows
+    keep the table."""
+    rng = np.random.default_rng(n % 1000 + len(value))
+    lens = [0, 1, 2, 3, 31, 32, 33, 64, 65, 100]        # one row of B per length and style
+    styles = ["spread", "left", "right"]
+    cols = []
+    for k in lens:
+        for s in styles:
+            c = rng.choice(min(n, 5000), k, replace=False) if s == "spread" else np.arange(k)
+            cols.append(np.sort(c if s != "right" else n - k + c))
+    rp = np.concatenate([[0], np.cumsum([c.size for c in cols])]).astype(np.int64)
+    col = np.concatenate(cols).astype(np.int32)
+    B = inputs.CSR(len(cols), n, rp, col, inputs.draw_values(rng, col.size, value))
+    size = np.diff(rp)
+    rows = []
+    for target in [33, 48, 63, 64, 65, 96, 127, 128, 129, 200]:
+        for _ in range(6):
+            pick, left = [], target
+            for k in rng.permutation(len(cols)):
+                if size[k] <= left:
+                    pick.append(k)
+                    left -= size[k]
+            rows.append(np.sort(pick))
+    rpA = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
+    colA = np.concatenate(rows).astype(np.int32)
+    A = inputs.CSR(len(rows), len(cols), rpA, colA, inputs.draw_values(rng, colA.size, value))
+    sr = 1 if value == "none" else 0
+    C = run(sg, A, B, semiring=sr)
+    R = oracle.spgemm(A, B, semiring="or_and" if sr else "plus_times")
+    assert_pattern_equal(C, R)
+    if value != "none":
+        assert np.array_equal(C.to_host()[2], R.val)
