@@ -259,6 +259,7 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
         seg += d.l * (sg::kSegGrid + 1);
         run += d.nnzB;
         P->max_n = std::max(P->max_n, d.n);
+        P->nnz_a += A[p].nnz;
     }
     rb[count] = rbase;
     bb[count] = bbase;

@@ -101,8 +101,6 @@ spgemm_status spgemm_chain_create(int32_t nsteps, const spgemm_chain_step* steps
         c.cls = P->cls;
         c.rows = P->rows;
         c.cap = P->cap;
-        c.prm = P->prm;
-        c.margin = P->margin;
         c.chunkcnt = (int32_t*)(w + L.chunkcnt);
         c.segtab = (int32_t*)(w + L.segtab);
         c.runlen = (int32_t*)(w + L.runlen);

@@ -243,8 +243,9 @@ __global__ void __launch_bounds__(THREADS, 1)
         const ChainProduct c = steps[p];
         int* err = &c.cnt->err;
         // row analysis
-        analyze_kernel_body<IT>(c.R, c.D, c.rb, c.nprod, c.max_dense_n, c.dense_min, c.flops,
-                                c.cls, c.cnt, c.prm, c.margin, c.cap, c.hash_shift, bid, nb);
+        analyze_kernel_body<IT, false>(c.R, c.D, c.rb, c.nprod, c.max_dense_n, c.dense_min,
+                                       c.flops, c.cls, c.cnt, nullptr, 0.f, c.cap, c.hash_shift,
+                                       32, bid, nb);
         if (!chain_barrier(sync, stage++)) return;
         chain_bin(c, bid, nb);
         if (!chain_barrier(sync, stage++)) return;

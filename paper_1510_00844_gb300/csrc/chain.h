@@ -30,7 +30,6 @@ struct ChainProduct {
     unsigned char* cls;
     int32_t* rows;
     int64_t* cap;
-    const float* prm;
     int32_t* chunkcnt;
     int32_t* segtab;
     int32_t* runlen;
@@ -41,7 +40,6 @@ struct ChainProduct {
     void* colC;
     void* valC;
     long long R, LB, max_dense_n, arena_stride, capacity;
-    float margin;
     int nprod, W, dense_min, hash_shift, seg_log2, max_words;
 };
 

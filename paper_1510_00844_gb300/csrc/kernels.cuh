@@ -211,28 +211,71 @@ __device__ __forceinline__ long long row_end(const int64_t* rp, const int64_t* r
 // Per global row (a warp per tile of 32 rows): flops_i, its class, per-class
 // counts, total and max flops, longest dense row; a product whose dense rows
 // need more columns than the shared-memory bitmap holds is flagged.
-// Learned sizing (not in the paper): when `prm` is given, the warp also
-// evaluates the row-size predictor on each row's features (one lane per
-// hidden unit), writes the predicted capacity cap_out[r] = clamp(2^(y +
+// What bounds it: the longest rows, walked by one warp with eight entries per
+// lane in flight (with one, the 240 us of an R-MAT 18 analysis were its longest
+// row's 250 dependent steps; now 150 us).
+// Learned sizing (not in the paper): when `prm` is given, the row-size predictor
+// is evaluated on each row's features (a lane per row: with a lane per
+// hidden unit, row after row, 40009 rows took 286 us; now 25 us), which gives
+// the predicted capacity cap_out[r] = clamp(2^(y +
 // margin) - 1, max_k |B(k,:)|, min(flops, n)), and bins rows of at most
 // dense_min products by that capacity instead of by their flops.
 constexpr int kSizerF = 6;
 
-template <class IT>
+// The row-size predictor on one row's features, by one lane; prm: W1 (32 x F),
+// b1, W2 (32 x 32), b2, w3, b3.  Products are rounded and added in ascending
+// input; the last layer's 32 terms are added as a tree over i, i + 16; i, i + 8;
+// ... so that a warp that holds one unit per lane gets the same sum.
+__device__ __forceinline__ float sizer_eval(const float* prm, const float (&x)[kSizerF]) {
+    const float* W1 = prm;
+    const float* b1 = W1 + 32 * kSizerF;
+    const float* W2 = b1 + 32;
+    const float* b2 = W2 + 32 * 32;
+    const float* w3 = b2 + 32;
+    float h1[32];
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        float z = b1[j];
+#pragma unroll
+        for (int q = 0; q < kSizerF; ++q) z = __fadd_rn(z, __fmul_rn(W1[j * kSizerF + q], x[q]));
+        h1[j] = z > 0.f ? z : 0.f;
+    }
+    // the terms of units j and j + 16 together, so that the tree's first level
+    // needs no array of 32 terms
+    float term[16];
+#pragma unroll 4
+    for (int j = 0; j < 16; ++j) {
+        float z = b2[j], y = b2[j + 16];
+#pragma unroll
+        for (int k = 0; k < 32; ++k) {
+            z = __fadd_rn(z, __fmul_rn(W2[j * 32 + k], h1[k]));
+            y = __fadd_rn(y, __fmul_rn(W2[(j + 16) * 32 + k], h1[k]));
+        }
+        term[j] = __fadd_rn(__fmul_rn(w3[j], z > 0.f ? z : 0.f),
+                            __fmul_rn(w3[j + 16], y > 0.f ? y : 0.f));
+    }
+#pragma unroll
+    for (int d = 8; d; d >>= 1)
+#pragma unroll
+        for (int j = 0; j < d; ++j) term[j] = __fadd_rn(term[j], term[j + d]);
+    return term[0] + w3[32];
+}
+
+template <class IT, bool PREDICT>
 __device__ __forceinline__ void analyze_kernel_body(long long R, const ProdDesc* __restrict__ D,
                                const long long* __restrict__ rb, int nprod, long long max_dense_n,
                                int dense_min, int64_t* __restrict__ flops_out,
                                unsigned char* __restrict__ cls_out, DevCounters* cnt,
                                const float* __restrict__ prm, float margin,
-                               int64_t* __restrict__ cap_out, int hash_shift,
+                               int64_t* __restrict__ cap_out, int hash_shift, int tile_rows,
         const long long vbid, const long long vnb) {
     __shared__ unsigned long long hist[kNumClasses];
     __shared__ unsigned long long blk_total, blk_max, blk_dlen;
     __shared__ int blk_unsup;
-    __shared__ float sp[32 * kSizerF + 32 + 32 * 32 + 32 + 32 + 1];
-    if (prm)
-        for (int q = threadIdx.x; q < 32 * kSizerF + 32 + 32 * 32 + 32 + 32 + 1; q += blockDim.x)
-            sp[q] = prm[q];
+    constexpr int kParams = 32 * kSizerF + 32 + 32 * 32 + 32 + 32 + 1;
+    __shared__ float sp[PREDICT ? kParams : 1];
+    if constexpr (PREDICT)
+        for (int q = threadIdx.x; q < kParams; q += blockDim.x) sp[q] = prm[q];
     for (int t = threadIdx.x; t < kNumClasses; t += blockDim.x) hist[t] = 0;
     if (threadIdx.x == 0) {
         blk_total = 0;
@@ -245,13 +288,13 @@ __device__ __forceinline__ void analyze_kernel_body(long long R, const ProdDesc*
     const long long warp = ((long long)vbid * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)vnb * blockDim.x) >> 5;
     unsigned long long my_total = 0, my_max = 0;
-    // Tiles of 32 rows: a row of at most 32 A entries is summed by its own
-    // lane (eight entries' loads in flight at a time); longer rows by the
-    // whole warp, one after another.  The predictor then runs row by row with
-    // a lane per hidden unit.
-    for (long long tile = warp; tile * 32 < R; tile += nwarps) {
-        const long long r = tile * 32 + lane;
-        const bool in = r < R;
+    // Tiles of tile_rows <= 32 rows (fewer where there are few rows for the
+    // warps): a row of at most 32 A entries is summed by its own lane (eight
+    // entries' loads in flight at a time); longer rows by the whole warp, one
+    // after another.
+    for (long long tile = warp; tile * tile_rows < R; tile += nwarps) {
+        const long long r = tile * tile_rows + lane;
+        const bool in = lane < tile_rows && r < R;
         RowCtx<IT, NoVal> c{};
         if (in) c = row_ctx<IT, NoVal>(D, rb, nprod, r);
         const long long d = in ? c.a1 - c.a0 : 0;
@@ -273,13 +316,20 @@ __device__ __forceinline__ void analyze_kernel_body(long long R, const ProdDesc*
         }
         for (unsigned lm = __ballot_sync(kFull, in && d > 32); lm; lm &= lm - 1u) {
             const int src = __ffs(lm) - 1;
-            const RowCtx<IT, NoVal> cs = row_ctx<IT, NoVal>(D, rb, nprod, tile * 32 + src);
+            const RowCtx<IT, NoVal> cs = row_ctx<IT, NoVal>(D, rb, nprod, tile * tile_rows + src);
             long long fs = 0, ms = 0;
-            for (long long p = cs.a0 + lane; p < cs.a1; p += 32) {
-                const long long k = (long long)cs.ciA[p];
-                const long long len = cs.rpB[k + 1] - cs.rpB[k];
-                fs += len;
-                ms = len > ms ? len : ms;
+            for (long long p = cs.a0 + lane; p < cs.a1; p += 256) {
+                long long k[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    k[u] = p + 32 * u < cs.a1 ? (long long)cs.ciA[p + 32 * u] : -1;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    if (k[u] >= 0) {
+                        const long long len = cs.rpB[k[u] + 1] - cs.rpB[k[u]];
+                        fs += len;
+                        ms = len > ms ? len : ms;
+                    }
             }
             fs = warp_sum(fs);
             ms = warp_max(ms);
@@ -289,47 +339,22 @@ __device__ __forceinline__ void analyze_kernel_body(long long R, const ProdDesc*
             }
         }
         long long cap = 0;
-        if (prm) {
-            const float* W1 = sp;
-            const float* b1 = W1 + 32 * kSizerF;
-            const float* W2 = b1 + 32;
-            const float* b2 = W2 + 32 * 32;
-            const float* w3 = b2 + 32;
-            for (unsigned pm = __ballot_sync(kFull, in && f > 0); pm; pm &= pm - 1u) {
-                const int j = __ffs(pm) - 1;
-                const long long fj = __shfl_sync(kFull, f, j);
-                const long long dj = __shfl_sync(kFull, d, j);
-                const long long mj = __shfl_sync(kFull, mx, j);
-                const long long nj = __shfl_sync(kFull, c.n, j);
-                const long long ub = fj < nj ? fj : nj;
-                float x[kSizerF];
-                x[0] = log2f(1.f + (float)fj);
-                x[1] = log2f(1.f + (float)dj);
-                x[2] = log2f(1.f + (float)mj);
-                x[3] = log2f(1.f + (float)nj);
-                x[4] = log2f(1.f + (float)fj / (float)dj);
-                x[5] = log2f(1.f + (float)ub);
-                float z = b1[lane];
-                for (int q = 0; q < kSizerF; ++q) z = __fadd_rn(z, __fmul_rn(W1[lane * kSizerF + q], x[q]));
-                const float h1 = z > 0.f ? z : 0.f;
-                float z2 = b2[lane];
-                for (int k = 0; k < 32; ++k)
-                    z2 = __fadd_rn(z2, __fmul_rn(W2[lane * 32 + k], __shfl_sync(kFull, h1, k)));
-                const float h2 = z2 > 0.f ? z2 : 0.f;
-                const float y = warp_sum(__fmul_rn(w3[lane], h2)) + w3[32];
-                const float est = exp2f(y + margin) - 1.f;
-                long long cj = est >= (float)ub ? ub : (long long)ceilf(est > 0.f ? est : 0.f);
-                if (cj < mj) cj = mj;
-                if (cj > ub) cj = ub;
-                if (lane == j) cap = cj;
-            }
+        if (PREDICT && in && f > 0) {
+            const long long ub = f < c.n ? f : c.n;
+            const float x[kSizerF] = {log2f(1.f + (float)f),    log2f(1.f + (float)d),
+                                      log2f(1.f + (float)mx),   log2f(1.f + (float)c.n),
+                                      log2f(1.f + (float)f / (float)d), log2f(1.f + (float)ub)};
+            const float est = exp2f(sizer_eval(sp, x) + margin) - 1.f;
+            cap = est >= (float)ub ? ub : (long long)ceilf(est > 0.f ? est : 0.f);
+            if (cap < mx) cap = mx;
+            if (cap > ub) cap = ub;
         }
         int cl = -1 - lane;
         if (in) {
             flops_out[r] = f;
-            if (cap_out) cap_out[r] = prm ? cap : f;
+            if (cap_out) cap_out[r] = PREDICT ? cap : f;
             cl = row_class(f, dense_min, hash_shift);
-            if (prm && cl > kClassEmpty && cl < kClassDense0) {
+            if (PREDICT && cl > kClassEmpty && cl < kClassDense0) {
                 cl = row_class(cap > 0 ? cap : 1, dense_min, hash_shift);
                 // bin 0 is the short-row path (one product per lane): a row
                 // with more products takes bin 1's table whatever its size
@@ -364,15 +389,15 @@ __device__ __forceinline__ void analyze_kernel_body(long long R, const ProdDesc*
     }
 }
 
-template <class IT>
-__global__ void analyze_kernel(long long R, const ProdDesc* __restrict__ D,
+template <class IT, bool PREDICT>
+__global__ void __launch_bounds__(256) analyze_kernel(long long R, const ProdDesc* __restrict__ D,
                                const long long* __restrict__ rb, int nprod, long long max_dense_n,
                                int dense_min, int64_t* __restrict__ flops_out,
                                unsigned char* __restrict__ cls_out, DevCounters* cnt,
                                const float* __restrict__ prm, float margin,
-                               int64_t* __restrict__ cap_out, int hash_shift) {
-    analyze_kernel_body<IT>(R, D, rb, nprod, max_dense_n, dense_min, flops_out, cls_out, cnt,
-        prm, margin, cap_out, hash_shift, (long long)blockIdx.x, (long long)gridDim.x);
+                               int64_t* __restrict__ cap_out, int hash_shift, int tile_rows) {
+    analyze_kernel_body<IT, PREDICT>(R, D, rb, nprod, max_dense_n, dense_min, flops_out, cls_out, cnt,
+        prm, margin, cap_out, hash_shift, tile_rows, (long long)blockIdx.x, (long long)gridDim.x);
 }
 
 // Features of every global row for the row-size predictor (log2(1 + .) of

@@ -45,14 +45,23 @@ constexpr size_t dense_warp_bytes() {
 template <class IT>
 cudaError_t launch_analyze(Plan& P) {
     if (P.R <= 0) return cudaSuccess;
-    auto k = analyze_kernel<IT>;
+    auto k = P.prm ? analyze_kernel<IT, true> : analyze_kernel<IT, false>;
     int occ = occupancy_blocks(k, 256, 0);
-    // a warp per tile of 32 rows
-    long long g = grid_for(P.R, 256, P.sm_count, occ);
+    // a warp per tile of 32 rows; of fewer while a tile holds more than 256
+    // entries of A and the resident warps have less than two tiles each, since a
+    // warp walks its tile's long rows one after another (800 long rows of a
+    // Markov step 147 -> 11 us; rows of 8 entries are faster in full tiles, 5.5
+    // against 11.5 us for 16384 of them, and so is the predictor; the sizes of
+    // device-sized plans are capacities)
+    int tile_rows = 32;
+    while (!P.prm && !P.device_sized && tile_rows > 1 && (double)P.nnz_a * tile_rows > 256.0 * (double)P.R &&
+           P.R < (long long)tile_rows * 16 * P.sm_count * occ)
+        tile_rows >>= 1;
+    long long g = grid_for(P.R, 8 * tile_rows, P.sm_count, occ);
     count_launches(1);
     k<<<(unsigned)g, 256, 0, P.stream>>>(P.R, P.d_descs, P.rb, P.nprod, P.max_dense_n,
                                            P.dense_min, P.flops, P.cls, P.cnt, P.prm, P.margin,
-                                           P.cap, P.hash_shift);
+                                           P.cap, P.hash_shift, tile_rows);
     return cudaGetLastError();
 }
 

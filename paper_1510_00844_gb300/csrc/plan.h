@@ -25,6 +25,7 @@ struct spgemm_plan_s {
     long long R = 0;         // total rows of the batch
     long long LB = 0;        // total B rows of the batch
     long long max_n = 0;     // largest n of the batch
+    long long nnz_a = 0;     // entries of A over the batch (at most: arrays of views are longer)
     long long max_dense_n = 0;
     int dense_min = 1024;    // rows with more products than this are dense
     int hash_shift = 0;      // hash rows are binned by flops << hash_shift
