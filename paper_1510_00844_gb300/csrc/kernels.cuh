@@ -1412,6 +1412,329 @@ __global__ void __launch_bounds__(WARPS * 32)
         vC, err, rowend, overflow, overflow_count, (long long)blockIdx.x, (long long)gridDim.x);
 }
 
+// One run of a batch of A entries whose products are flattened: product f of
+// the run sits at B position off + f, and is scaled by a = A(i,k).
+template <class V>
+struct __align__(16) DenseRun {
+    long long off;
+    V a;
+};
+
+// ------------------------- rows of 129 to 1024 products, ranked by a bitmap
+// Hash bins 2 and 3 in products of at most rank_max_n columns.  A block of four
+// warps takes a row; product f of the row (ascending k) sits in warp (f / 32) %
+// 4, lane f % 32, item f / 128.  The products set the bits of their columns;
+// the set bits before a column are its place in C(i,:), so nothing is hashed or
+// sorted.  The first product of every place (the smallest f, by atomicMin)
+// stores its value; the others, few in a sparse row, are listed in ascending f
+// and added by one warp in that order.
+// What bounds it: instructions, at 24 to 28 warps per SM.  A warp with a table
+// per row (25 KB for float64) held 12 warps and took 9.7 instructions per
+// product: 64 uneven Erdos-Renyi products in float32 (up to 65536 columns),
+// rows of 513 to 1024 products 6.25 -> 2.34 ms, their counts 1.45 -> 0.91 ms.
+constexpr int kRankWarps = 4;
+constexpr int kRankItems = 8;
+constexpr int kRankMost = 32 * kRankWarps * kRankItems;   // products of a row
+static_assert(kRankMost >= hash_bin_flops(kNumHashBins - 1), "a hash row fits");
+// Most columns for which the bitmap beats the table, by bin and pass: clearing
+// and counting it costs the same whatever the row holds.
+__host__ __device__ constexpr long long rank_max_n(int bin, bool count) {
+    return bin == 3 ? 262144 : bin == 2 ? (count ? 16384 : 32768) : 0;
+}
+
+// Words of the bitmap of n columns: each warp takes whole groups of 128.
+__host__ __device__ constexpr int rank_words(long long n) {
+    return (int)((n + 128 * 32 * kRankWarps - 1) / (128 * 32 * kRankWarps)) * 128 * kRankWarps;
+}
+
+// Shared memory: the column map (bits, then the set bits before every word;
+// its room is the list of later products afterwards), places' first products
+// and then columns, accumulators, and a table of runs per warp.
+template <class V>
+struct RankSmem {
+    static constexpr size_t kList = kRankMost * (sizeof(int) + (VOps<V>::has_val ? sizeof(V) : 0));
+    size_t before, tag, acc, runs, total;
+    __host__ __device__ explicit RankSmem(long long n, bool count) {
+        before = (size_t)rank_words(n) * sizeof(unsigned);
+        const size_t map = before + (count ? 0 : (size_t)rank_words(n) * sizeof(unsigned short));
+        tag = ((count || map > kList ? map : kList) + 15) / 16 * 16;
+        acc = tag + (count ? 0 : kRankMost * sizeof(unsigned));
+        runs = acc + (!count && VOps<V>::has_val ? kRankMost * sizeof(V) : 0);
+        total = runs + kRankWarps * 32 * sizeof(DenseRun<V>);
+    }
+};
+
+// Columns (-1: none) and values of this lane's products of the row.
+template <class IT, class V, bool VALS>
+__device__ __forceinline__ void rank_gather(const RowCtx<IT, V>& c, int w, int (&col)[kRankItems],
+                                            V (&v)[kRankItems], DenseRun<V>* runs) {
+    const int lane = lane_id();
+#pragma unroll
+    for (int t = 0; t < kRankItems; ++t) {
+        col[t] = -1;
+        v[t] = VOps<V>::init();
+    }
+    int have = 0;
+    for (long long b = c.a0; b < c.a1; b += 32) {
+        const int nb = (int)min(32LL, c.a1 - b);
+        long long lo = 0;
+        int len = 0;
+        DenseRun<V> run{};
+        if (lane < nb) {
+            const long long k = (long long)c.ciA[b + lane];
+            lo = c.rpB[k];
+            len = (int)min(c.rpB[k + 1] - lo, (long long)kRankMost);
+            if constexpr (VALS) run.a = load_val(c.vA, b + lane);
+        }
+        const int incl = warp_incl_scan(len);
+        const int tot = min(__shfl_sync(kFull, incl, 31), kRankMost - have);
+        if (tot <= 0) continue;
+        const int start = have + incl - len;
+        const unsigned some = __ballot_sync(kFull, len > 0);
+        run.off = lo - start;
+        __syncwarp();   // the table's last use is over
+        if (len > 0) runs[__popc(some & lanemask_lt())] = run;
+        __syncwarp();
+#pragma unroll
+        for (int t = 0; t < kRankItems; ++t) {
+            const int w0 = 32 * (kRankWarps * t + w);
+            if (w0 >= have + tot || w0 + 32 <= have) continue;
+            // the run of product f: the runs that start at or before it
+            const unsigned M = __reduce_or_sync(
+                kFull, len > 0 && start >= w0 && start < w0 + 32 ? 1u << (start - w0) : 0u);
+            const int e = __popc(__ballot_sync(kFull, len > 0 && start < w0)) +
+                          __popc(M & lanemask_le()) - 1;
+            const int f = w0 + lane;
+            if (f >= have && f < have + tot) {
+                const DenseRun<V> x = runs[e];
+                const long long q = x.off + f;
+                col[t] = (int)c.ciB[q];
+                if constexpr (VALS) v[t] = VOps<V>::mul(x.a, load_val(c.vB, q));
+            }
+        }
+        have += tot;
+    }
+}
+
+// Set bits before every word of the map and their total; warp w owns the words
+// [w, w + 1) * nwords / 4, four per lane and step.  Two barriers; the last one
+// covers the words' counts too.
+__device__ __forceinline__ int rank_prefix(const unsigned* bits, unsigned short* before, int nwords,
+                                           int w, int* part) {
+    const int lane = lane_id();
+    const int per = nwords / kRankWarps;
+    const uint4* b4 = reinterpret_cast<const uint4*>(bits + w * per);
+    ushort4* p4 = reinterpret_cast<ushort4*>(before + w * per);
+    int sum = 0;
+    for (int t = lane; t < per / 4; t += 32) {
+        const uint4 x = b4[t];
+        sum += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+    }
+    sum = warp_sum(sum);
+    if (lane == 0) part[w] = sum;
+    __syncthreads();
+    int base = 0, total = 0;
+#pragma unroll
+    for (int u = 0; u < kRankWarps; ++u) {
+        base += u < w ? part[u] : 0;
+        total += part[u];
+    }
+    for (int t = lane; t < per / 4; t += 32) {
+        const uint4 x = b4[t];
+        const int p0 = __popc(x.x), p1 = p0 + __popc(x.y), p2 = p1 + __popc(x.z),
+                  p3 = p2 + __popc(x.w);
+        const int incl = warp_incl_scan(p3);
+        const int at = base + incl - p3;
+        p4[t] = make_ushort4((unsigned short)at, (unsigned short)(at + p0),
+                             (unsigned short)(at + p1), (unsigned short)(at + p2));
+        base += __shfl_sync(kFull, incl, 31);
+    }
+    __syncthreads();
+    return total;
+}
+
+__device__ __forceinline__ void rank_clear(unsigned* bits, int nwords) {
+    uint4* b4 = reinterpret_cast<uint4*>(bits);
+    for (int t = threadIdx.x; t < nwords / 4; t += blockDim.x) b4[t] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+template <class IT>
+__global__ void __launch_bounds__(32 * kRankWarps)
+    symbolic_rank_kernel(const ProdDesc* __restrict__ D, const long long* __restrict__ rb,
+                         int nprod, const int32_t* __restrict__ rows, const DevCounters* cnt,
+                         int cls, long long max_n, int64_t* __restrict__ rowcnt) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int total;
+    const RankSmem<NoVal> L(max_n, true);
+    unsigned* bits = reinterpret_cast<unsigned*>(smem_raw);
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    DenseRun<NoVal>* runs = reinterpret_cast<DenseRun<NoVal>*>(smem_raw + L.runs) + 32 * w;
+    rank_clear(bits, rank_words(max_n));
+    if (threadIdx.x == 0) total = 0;
+    __syncthreads();
+    const long long nrows = (long long)cnt->class_count[cls];
+    const int32_t* crow = rows + cnt->class_off[cls];
+    for (long long rr = blockIdx.x; rr < nrows; rr += gridDim.x) {
+        const long long r = crow[rr];
+        const RowCtx<IT, NoVal> c = row_ctx<IT, NoVal>(D, rb, nprod, r);
+        int col[kRankItems];
+        NoVal v[kRankItems];
+        rank_gather<IT, NoVal, false>(c, w, col, v, runs);
+#pragma unroll
+        for (int t = 0; t < kRankItems; ++t)
+            if (col[t] >= 0) atomicOr(&bits[col[t] >> 5], 1u << (col[t] & 31));
+        __syncthreads();
+        int sum = 0;
+        uint4* b4 = reinterpret_cast<uint4*>(bits);
+        for (int t = threadIdx.x; t < rank_words(c.n) / 4; t += blockDim.x) {
+            const uint4 x = b4[t];
+            sum += __popc(x.x) + __popc(x.y) + __popc(x.z) + __popc(x.w);
+            b4[t] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        sum = warp_sum(sum);
+        if (lane == 0 && sum) atomicAdd(&total, sum);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            rowcnt[r] = total;
+            total = 0;
+        }
+    }
+}
+
+template <class IT, class V>
+__global__ void __launch_bounds__(32 * kRankWarps)
+    numeric_rank_kernel(const ProdDesc* __restrict__ D, const long long* __restrict__ rb,
+                        int nprod, const int32_t* __restrict__ rows, const DevCounters* cnt,
+                        int cls, long long max_n, const int64_t* __restrict__ rpC, long long cap,
+                        IT* __restrict__ ciC, V* __restrict__ vC, int* err,
+                        int64_t* __restrict__ rowend, int32_t* __restrict__ overflow,
+                        unsigned* overflow_count) {
+    constexpr bool HV = VOps<V>::has_val;
+    constexpr bool kPlain = std::is_same<V, double>::value || std::is_same<V, float>::value ||
+                            std::is_same<V, int64_t>::value;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ int part[32];
+    const RankSmem<V> L(max_n, false);
+    unsigned* bits = reinterpret_cast<unsigned*>(smem_raw);
+    unsigned short* before = reinterpret_cast<unsigned short*>(smem_raw + L.before);
+    V* list_v = reinterpret_cast<V*>(smem_raw);
+    int* list_s = reinterpret_cast<int*>(smem_raw + (HV ? kRankMost * sizeof(V) : 0));
+    unsigned* tag = reinterpret_cast<unsigned*>(smem_raw + L.tag);
+    V* acc = reinterpret_cast<V*>(smem_raw + L.acc);
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    DenseRun<V>* runs = reinterpret_cast<DenseRun<V>*>(smem_raw + L.runs) + 32 * w;
+    rank_clear(bits, rank_words(max_n));
+    for (int t = threadIdx.x; t < kRankMost; t += blockDim.x) tag[t] = 0xffffffffu;
+    __syncthreads();
+    const long long nrows = (long long)cnt->class_count[cls];
+    const int32_t* crow = rows + cnt->class_off[cls];
+    for (long long rr = blockIdx.x; rr < nrows; rr += gridDim.x) {
+        const long long r = crow[rr];
+        const RowCtx<IT, V> c = row_ctx<IT, V>(D, rb, nprod, r);
+        const long long out = rpC[r];
+        const long long room = rpC[r + 1] - out;
+        int col[kRankItems];
+        V v[kRankItems];
+        rank_gather<IT, V, HV>(c, w, col, v, runs);
+#pragma unroll
+        for (int t = 0; t < kRankItems; ++t)
+            if (col[t] >= 0) atomicOr(&bits[col[t] >> 5], 1u << (col[t] & 31));
+        __syncthreads();
+        int nwords = rank_words(c.n);
+        const int total = rank_prefix(bits, before, nwords, w, part);
+        // slot mode: a row that outgrows its slot is listed for an exact re-run
+        bool write = true;
+        if (rowend != nullptr) {
+            write = total <= room;
+            if (threadIdx.x == 0) {
+                if (!write) overflow[atomicAdd(overflow_count, 1u)] = (int32_t)r;
+                rowend[r] = write ? out + total : -1;
+            }
+        } else if (threadIdx.x == 0) {
+            if (total != room) atomicExch(err, (int)kDevCountMismatch);
+            if (out + room > cap) atomicExch(err, (int)kDevCapacity);
+        }
+        if constexpr (HV) {
+            int slot[kRankItems];
+#pragma unroll
+            for (int t = 0; t < kRankItems; ++t) {
+                slot[t] = -1;
+                if (col[t] >= 0) {
+                    slot[t] = before[col[t] >> 5] +
+                              __popc(bits[col[t] >> 5] & ~(0xffffffffu << (col[t] & 31)));
+                    atomicMin(&tag[slot[t]], (unsigned)(32 * (kRankWarps * t + w) + lane));
+                }
+            }
+            __syncthreads();
+            bool later[kRankItems];   // not the first product of its place
+            bool any = false;
+#pragma unroll
+            for (int t = 0; t < kRankItems; ++t) {
+                later[t] = slot[t] >= 0 &&
+                           tag[slot[t]] != (unsigned)(32 * (kRankWarps * t + w) + lane);
+                any = any || later[t];
+            }
+            any = __syncthreads_or(any);
+#pragma unroll
+            for (int t = 0; t < kRankItems; ++t)
+                if (slot[t] >= 0 && !later[t]) {
+                    tag[slot[t]] = (unsigned)col[t];
+                    // the identity plus x is x, bit for bit, for (+, x)
+                    if constexpr (kPlain) acc[slot[t]] = v[t];
+                    else acc[slot[t]] = VOps<V>::add(VOps<V>::init(), v[t]);
+                }
+            if (any) {
+                nwords = rank_words(max_n);   // the list may lie over all of the bits
+                // item t of warp w comes t * 4 + w-th
+                static_assert(kRankItems * kRankWarps == 32, "a lane per group of products");
+#pragma unroll
+                for (int t = 0; t < kRankItems; ++t) {
+                    const unsigned m = __ballot_sync(kFull, later[t]);
+                    if (lane == 0) part[kRankWarps * t + w] = __popc(m);
+                }
+                __syncthreads();
+                const int k = part[lane];
+                const int incl = warp_incl_scan(k);
+                const int nlist = __shfl_sync(kFull, incl, 31);
+#pragma unroll
+                for (int t = 0; t < kRankItems; ++t) {
+                    const int at = __shfl_sync(kFull, incl - k, kRankWarps * t + w);
+                    const unsigned m = __ballot_sync(kFull, later[t]);
+                    if (later[t]) {
+                        list_s[at + __popc(m & lanemask_lt())] = slot[t];
+                        list_v[at + __popc(m & lanemask_lt())] = v[t];
+                    }
+                }
+                __syncthreads();
+                if (w == 0)
+                    for (int x0 = 0; x0 < nlist; x0 += 32) {
+                        const bool valid = x0 + lane < nlist;
+                        ordered_add(acc, valid ? list_s[x0 + lane] : 0, valid,
+                                    valid ? list_v[x0 + lane] : VOps<V>::init());
+                    }
+            }
+            __syncthreads();
+        } else {
+            // the columns of the set bits, in order
+            for (int t = threadIdx.x; t < nwords; t += blockDim.x) {
+                unsigned p = before[t];
+                for (unsigned word = bits[t]; word; word &= word - 1u)
+                    tag[p++] = (unsigned)(32 * t + __ffs(word) - 1);
+            }
+            __syncthreads();
+        }
+        for (int x = threadIdx.x; x < total; x += blockDim.x) {
+            if (write && x < room && out + x < cap) {
+                ciC[out + x] = (IT)tag[x];
+                if constexpr (HV) vC[out + x] = acc[x];
+            }
+            tag[x] = 0xffffffffu;
+        }
+        rank_clear(bits, nwords);
+        __syncthreads();
+    }
+}
+
 // --------------------------------------------------- numeric: dense rows
 // Work units: a dense row's P column chunks (width W) are cut into G equal
 // segments (G in {1, 2, 4, ..., kSegGrid}, chosen per flops class so that a
@@ -1435,14 +1758,6 @@ struct __align__(16) DenseCursor {
     long long pos;
     int col;
     int rl;
-};
-
-// One run of a batch in the dense numeric kernel: the flattened product f
-// of the run sits at B position off + f, and is scaled by a = A(i,k).
-template <class V>
-struct __align__(16) DenseRun {
-    long long off;
-    V a;
 };
 
 // runlen[run_base + q] = number of entries from q to the end of q's column

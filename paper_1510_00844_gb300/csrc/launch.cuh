@@ -97,6 +97,46 @@ cudaError_t launch_kslice_bounds(const spgemm_csr& A, int c, int64_t* bounds, in
     return cudaGetLastError();
 }
 
+// Bins 2 and 3 are ranked by a bitmap where that is faster than the table.
+// Erdos-Renyi squares, float64, table and bitmap in us: 30 per column (bin 3),
+// numeric 352 and 57 at 8192 columns, 1949 and 445 at 65536, 4194 and 1381 at
+// 131072, 8464 and 5384 at 262144; counts 53 and 21, 327 and 148, 623 and 321,
+// 1214 and 935; 16 per column (bin 2), numeric 60 and 42 at 8192, 187 and 159 at
+// 32768, 350 and 335 at 65536 (float32 288 and 303; uneven batches up to 65536
+// columns 2540 and 3060); counts 33 and 29 at 16384, 56 and 60 at 32768.
+inline bool rank_bin(const Plan& P, int bin, bool count) {
+    return P.max_n <= rank_max_n(bin, count);
+}
+
+template <class IT>
+cudaError_t sym_rank_bin(Plan& P, int bin, long long nrows, int64_t* rowcnt) {
+    auto k = symbolic_rank_kernel<IT>;
+    const size_t smem = RankSmem<NoVal>(P.max_n, true).total;
+    cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
+    const int occ = occupancy_blocks(k, 32 * kRankWarps, smem);
+    count_launches(1);
+    k<<<(unsigned)class_grid(P, nrows, 1, occ), 32 * kRankWarps, smem, P.stream>>>(
+        P.d_descs, P.rb, P.nprod, P.rows, P.cnt, kClassHash0 + bin, P.max_n, rowcnt);
+    return cudaGetLastError();
+}
+
+template <class IT, class V>
+cudaError_t num_rank_bin(Plan& P, int bin, long long nrows, const int64_t* rpC, long long cap,
+                         IT* colC, V* valC, int64_t* rowend, int32_t* overflow,
+                         unsigned* overflow_count) {
+    auto k = numeric_rank_kernel<IT, V>;
+    const size_t smem = RankSmem<V>(P.max_n, false).total;
+    cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
+    const int occ = occupancy_blocks(k, 32 * kRankWarps, smem);
+    count_launches(1);
+    k<<<(unsigned)class_grid(P, nrows, 1, occ), 32 * kRankWarps, smem, P.stream>>>(
+        P.d_descs, P.rb, P.nprod, P.rows, P.cnt, kClassHash0 + bin, P.max_n, rpC, cap, colC, valC,
+        &P.cnt->err, rowend, overflow, overflow_count);
+    return cudaGetLastError();
+}
+
 template <class IT, int LOG2T, int WARPS>
 cudaError_t sym_hash_bin(Plan& P, int bin, int64_t* rowcnt) {
     using K = typename KeyT<IT>::type;
@@ -105,6 +145,7 @@ cudaError_t sym_hash_bin(Plan& P, int bin, int64_t* rowcnt) {
     if (!P.device_sized && nrows == 0) return cudaSuccess;
     if (P.device_sized && bin > 0 && (hash_bin_flops(bin - 1) >> P.hash_shift) >= P.dense_min)
         return cudaSuccess;
+    if (rank_bin(P, bin, true)) return sym_rank_bin<IT>(P, bin, nrows, rowcnt);
     auto k = symbolic_hash_kernel<IT, LOG2T, WARPS>;
     size_t smem = LOG2T == kShortLog2T ? 0 : (size_t)WARPS * (1u << LOG2T) * sizeof(K);
     cudaError_t e = allow_smem(k, smem);
@@ -196,6 +237,9 @@ cudaError_t num_hash_bin(Plan& P, int bin, const int64_t* rpC, long long cap, IT
     if (!P.device_sized && nrows == 0) return cudaSuccess;
     if (P.device_sized && bin > 0 && (hash_bin_flops(bin - 1) >> P.hash_shift) >= P.dense_min)
         return cudaSuccess;
+    if (rank_bin(P, bin, false))
+        return num_rank_bin<IT, V>(P, bin, nrows, rpC, cap, colC, valC, rowend, overflow,
+                                   overflow_count);
     auto k = numeric_hash_kernel<IT, V, LOG2T, WARPS>;
     constexpr size_t vb = VOps<V>::has_val ? sizeof(V) : 0;
     size_t smem = LOG2T == kShortLog2T

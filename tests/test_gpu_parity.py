@@ -485,3 +485,53 @@ def test_rows_of_33_to_128_products(sg, n, value):
     assert_pattern_equal(C, R)
     if value != "none":
         assert np.array_equal(C.to_host()[2], R.val)
+
+
+@pytest.mark.parametrize("n,value", [(2000, "u01_f64"), (16384, "none"), (16385, "u11_f32"),
+                                     (32768, "int"), (32769, "u01_f64"), (262144, "u01_f64"),
+                                     (262144, "none"), (262145, "int")])
+def test_rows_of_129_to_1024_products(sg, n, value):
+    """Rows at the edges of the bitmap-ranked bins, on both sides of the widths
+    up to which they are ranked: all columns distinct, every column hit by many
+    A entries, and single products over a thousand A entries between empty
+    rows of B; the last column among them."""
+    rng = np.random.default_rng(n % 1000 + len(value))
+    lens = [0] * 40 + [1] * 1100 + [7, 31, 32, 33, 64, 100, 128, 129, 300, 512, 1024]
+    cols = []
+    for t, k in enumerate(lens):
+        if t % 3 == 0:
+            c = rng.choice(n, k, replace=False)
+        elif t % 3 == 1:
+            c = np.arange(k)
+        else:
+            c = n - k + np.arange(k)
+        cols.append(np.sort(c))
+    order = rng.permutation(len(lens))
+    cols = [cols[t] for t in order]
+    size = np.array([c.size for c in cols])
+    B = inputs.CSR(len(cols), n, np.concatenate([[0], np.cumsum(size)]).astype(np.int64),
+                   np.concatenate(cols).astype(np.int32),
+                   inputs.draw_values(rng, int(size.sum()), value))
+    rows = []
+    for target in [128, 129, 130, 511, 512, 513, 1000, 1023, 1024, 1025]:
+        for single in (False, True):
+            for _ in range(3):
+                pick, left = [], target
+                for k in rng.permutation(len(cols)):
+                    if size[k] <= left and (not single or size[k] <= 1):
+                        pick.append(k)
+                        left -= size[k]
+                    if left == 0:
+                        break
+                rows.append(np.sort(pick))
+    colA = np.concatenate(rows).astype(np.int32)
+    rpA = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
+    A = inputs.CSR(len(rows), len(cols), rpA, colA, inputs.draw_values(rng, colA.size, value))
+    sr = 1 if value == "none" else 0
+    C = run(sg, A, B, semiring=sr)
+    R = oracle.spgemm(A, B, semiring="or_and" if sr else "plus_times")
+    assert_pattern_equal(C, R)
+    if value == "u11_f32":
+        assert_values_close(C, R, A, B, "f32")
+    elif value != "none":
+        assert np.array_equal(C.to_host()[2], R.val)
