@@ -502,7 +502,6 @@ spgemm_status spgemm_symbolic(spgemm_plan_t P, void* ws, size_t ws_bytes, int64_
     if (st != SPGEMM_OK) return st;
     cudaStream_t s = P->stream;
     unsigned char* w = (unsigned char*)ws;
-    SG_CUDA(cudaMemsetAsync(rowptrC + P->R, 0, sizeof(int64_t), s), "symbolic: memset");
     cudaError_t e = P->it == SPGEMM_INDEX_I32 ? sg::launch_symbolic<int32_t>(*P, w, rowptrC)
                                               : sg::launch_symbolic<int64_t>(*P, w, rowptrC);
     if (e != cudaSuccess) return cuda_fail(e, "symbolic");
@@ -556,7 +555,6 @@ spgemm_status spgemm_execute(spgemm_plan_t P, void* ws, size_t ws_bytes, int64_t
     SG_CUDA(cudaMemsetAsync(P->cnt, 0, sizeof(sg::DevCounters), s), "execute: memset");
     cudaError_t e = P->it == SPGEMM_INDEX_I32 ? sg::launch_analyze<int32_t>(*P) : sg::launch_analyze<int64_t>(*P);
     if (e == cudaSuccess) e = sg::launch_binning(*P);
-    if (e == cudaSuccess) e = cudaMemsetAsync(rowptrC + P->R, 0, sizeof(int64_t), s);
     if (e == cudaSuccess)
         e = P->it == SPGEMM_INDEX_I32 ? sg::launch_symbolic<int32_t>(*P, w, rowptrC)
                                       : sg::launch_symbolic<int64_t>(*P, w, rowptrC);

@@ -4,24 +4,8 @@
 
 namespace sg {
 
-// Class offsets (exclusive scan of the counts) and the dense work-unit
-// prefix, one thread.
 __global__ void class_offsets_kernel(DevCounters* cnt, int seg_log2) {
-    cnt->seg_log2 = seg_log2;
-    unsigned long long s = 0;
-    for (int c = 0; c < kNumClasses; ++c) {
-        cnt->class_cursor[c] = s;
-        cnt->class_off[c] = s;
-        s += cnt->class_count[c];
-    }
-    cnt->class_off[kNumClasses] = s;
-    unsigned long long u = 0;
-    for (int t = 0; t < kMaxDenseClasses; ++t) {
-        cnt->unit_begin[t] = u;
-        u += cnt->class_count[kClassDense0 + t] *
-             (unsigned long long)dense_class_segments(t, seg_log2);
-    }
-    cnt->unit_begin[kMaxDenseClasses] = u;
+    class_offsets(cnt, seg_log2);
 }
 
 // Scatter global row ids into their class segment (order inside a class is
@@ -50,24 +34,33 @@ __global__ void bin_rows_kernel(long long R, const unsigned char* __restrict__ c
 }
 
 // ------------------------------------------------------------------ scan
-// In-place exclusive scan of int64 x[0..N).  Tiles of 4096 (256 x 16).
+// In-place exclusive scan of int64 x[0..N).  Tiles of 4096: a warp takes 512
+// consecutive entries, 16 per lane, all loaded at once (a tile taken 256
+// entries at a time, with four barriers each, was 8.7 us of the 0.18 ms of a
+// small product; now 3).  One tile takes one kernel, up to kScanDirect tiles
+// two (every block adds up the sums of the tiles before its own), more three.
+constexpr long long kScanDirect = 2048;
 
-__global__ void scan_reduce_kernel(const int64_t* __restrict__ x, long long N,
-                                   int64_t* __restrict__ part) {
+__global__ void __launch_bounds__(kScanThreads)
+    scan_reduce_kernel(const int64_t* __restrict__ x, long long N, int64_t* __restrict__ part) {
     __shared__ long long ws[kScanThreads / 32];
     long long base = (long long)blockIdx.x * kScanTile;
-    long long s = 0;
+    long long v[kScanItems];
+#pragma unroll
     for (int t = 0; t < kScanItems; ++t) {
-        long long idx = base + (long long)t * kScanThreads + threadIdx.x;
-        if (idx < N) s += x[idx];
+        const long long idx = base + (long long)t * kScanThreads + threadIdx.x;
+        v[t] = idx < N ? x[idx] : 0;
     }
+    long long s = 0;
+#pragma unroll
+    for (int t = 0; t < kScanItems; ++t) s += v[t];
     s = warp_sum(s);
     if (lane_id() == 0) ws[threadIdx.x >> 5] = s;
     __syncthreads();
     if (threadIdx.x < 32) {
-        long long v = threadIdx.x < kScanThreads / 32 ? ws[threadIdx.x] : 0;
-        v = warp_sum(v);
-        if (threadIdx.x == 0) part[blockIdx.x] = v;
+        long long w = threadIdx.x < kScanThreads / 32 ? ws[threadIdx.x] : 0;
+        w = warp_sum(w);
+        if (threadIdx.x == 0) part[blockIdx.x] = w;
     }
 }
 
@@ -97,41 +90,41 @@ __global__ void scan_partials_kernel(int64_t* part, long long nparts) {
     }
 }
 
-__global__ void scan_apply_kernel(int64_t* __restrict__ x, long long N,
-                                  const int64_t* __restrict__ part) {
-    __shared__ long long ws[kScanThreads / 32];
-    __shared__ long long carry;
-    long long base = (long long)blockIdx.x * kScanTile;
-    if (threadIdx.x == 0) carry = part[blockIdx.x];
-    __syncthreads();
-    for (int t = 0; t < kScanItems; ++t) {
-        long long idx = base + (long long)t * kScanThreads + threadIdx.x;
-        long long v = idx < N ? x[idx] : 0;
-        long long inc = warp_incl_scan(v);
-        if (lane_id() == 31) ws[threadIdx.x >> 5] = inc;
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            long long w = threadIdx.x < kScanThreads / 32 ? ws[threadIdx.x] : 0;
-            long long wi = warp_incl_scan(w);
-            if (threadIdx.x < kScanThreads / 32) ws[threadIdx.x] = wi - w;
-        }
-        __syncthreads();
-        long long excl = carry + ws[threadIdx.x >> 5] + inc - v;
-        if (idx < N) x[idx] = excl;
-        __syncthreads();
-        if (threadIdx.x == kScanThreads - 1) carry = excl + v;
-        __syncthreads();
+// part: the tiles' sums (direct), or the sums of the tiles before each.
+__global__ void __launch_bounds__(kScanThreads)
+    scan_apply_kernel(int64_t* __restrict__ x, long long N, const int64_t* __restrict__ part,
+                      bool direct) {
+    constexpr int kWarps = kScanThreads / 32;
+    __shared__ long long ws[kWarps], before[kWarps];
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    const long long base = (long long)blockIdx.x * kScanTile + (long long)w * 32 * kScanItems + lane;
+    long long v[kScanItems];
+#pragma unroll
+    for (int t = 0; t < kScanItems; ++t) v[t] = base + 32 * t < N ? x[base + 32 * t] : 0;
+    long long prev = 0;
+    if (direct)
+        for (long long u = threadIdx.x; u < blockIdx.x; u += kScanThreads) prev += part[u];
+    else if (threadIdx.x == 0)
+        prev = part[blockIdx.x];
+    long long s = 0;
+#pragma unroll
+    for (int t = 0; t < kScanItems; ++t) s += v[t];
+    s = warp_sum(s);
+    prev = warp_sum(prev);
+    if (lane == 0) {
+        ws[w] = s;
+        before[w] = prev;
     }
-}
-
-// Empty rows: count 0.
-__global__ void zero_rows_kernel(const int32_t* __restrict__ rows, const DevCounters* cnt,
-                                 int64_t* __restrict__ rowcnt) {
-    const long long nrows = (long long)cnt->class_count[kClassEmpty];
-    const int32_t* erow = rows + cnt->class_off[kClassEmpty];
-    for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < nrows;
-         r += (long long)gridDim.x * blockDim.x)
-        rowcnt[erow[r]] = 0;
+    __syncthreads();
+    long long carry = 0;
+#pragma unroll
+    for (int u = 0; u < kWarps; ++u) carry += before[u] + (u < w ? ws[u] : 0);
+#pragma unroll
+    for (int t = 0; t < kScanItems; ++t) {
+        const long long incl = warp_incl_scan(v[t]);
+        if (base + 32 * t < N) x[base + 32 * t] = carry + incl - v[t];
+        carry += __shfl_sync(kFull, incl, 31);
+    }
 }
 
 // Relative row pointers of every product: out[out_base_p + i] = g[rb_p + i] - g[rb_p].
@@ -153,19 +146,17 @@ __global__ void product_rowptr_kernel(long long R, const long long* __restrict__
 
 cudaError_t launch_class_offsets(Plan& P) {
     count_launches(1);
-    class_offsets_kernel<<<1, 1, 0, P.stream>>>(P.cnt, P.seg_log2);
+    class_offsets_kernel<<<1, 32, 0, P.stream>>>(P.cnt, P.seg_log2);
     return cudaGetLastError();
 }
 
+// The row analysis has formed the class offsets (there is none without rows).
 cudaError_t launch_binning(Plan& P) {
     const long long R = P.R;
+    if (R <= 0) return launch_class_offsets(P);
+    int blocks = (int)std::max<long long>(1, std::min<long long>((R + 1023) / 1024, (long long)P.sm_count * 4));
     count_launches(1);
-    class_offsets_kernel<<<1, 1, 0, P.stream>>>(P.cnt, P.seg_log2);
-    if (R > 0) {
-        int blocks = (int)std::max<long long>(1, std::min<long long>((R + 1023) / 1024, (long long)P.sm_count * 4));
-        count_launches(1);
-        bin_rows_kernel<<<blocks, 256, 0, P.stream>>>(R, P.cls, P.rows, P.cnt);
-    }
+    bin_rows_kernel<<<blocks, 256, 0, P.stream>>>(R, P.cls, P.rows, P.cnt);
     return cudaGetLastError();
 }
 
@@ -177,19 +168,17 @@ size_t scan_temp_bytes(long long N) {
 cudaError_t launch_exclusive_scan(int64_t* x, long long N, int64_t* temp, cudaStream_t s) {
     if (N <= 0) return cudaSuccess;
     long long parts = (N + kScanTile - 1) / kScanTile;
+    const bool direct = parts <= kScanDirect;
+    if (parts > 1) {
+        count_launches(1);
+        scan_reduce_kernel<<<(unsigned)parts, kScanThreads, 0, s>>>(x, N, temp);
+    }
+    if (!direct) {
+        count_launches(1);
+        scan_partials_kernel<<<1, 1024, 0, s>>>(temp, parts);
+    }
     count_launches(1);
-    scan_reduce_kernel<<<(unsigned)parts, kScanThreads, 0, s>>>(x, N, temp);
-    count_launches(1);
-    scan_partials_kernel<<<1, 1024, 0, s>>>(temp, parts);
-    count_launches(1);
-    scan_apply_kernel<<<(unsigned)parts, kScanThreads, 0, s>>>(x, N, temp);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_zero_rows(const Plan& P, int64_t* rowcnt) {
-    int blocks = P.sm_count * 4;
-    count_launches(1);
-    zero_rows_kernel<<<blocks, 256, 0, P.stream>>>(P.rows, P.cnt, rowcnt);
+    scan_apply_kernel<<<(unsigned)parts, kScanThreads, 0, s>>>(x, N, temp, direct);
     return cudaGetLastError();
 }
 

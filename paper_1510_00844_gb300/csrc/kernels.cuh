@@ -76,7 +76,8 @@ struct DevCounters {
     int err;
     int unsupported;
     int seg_log2;                        // dense work-unit size of the plan
-    int pad[29];
+    unsigned blocks_done;                // of the row analysis
+    int pad[28];
 };
 
 // Product owning global row r: the largest p with rb[p] <= r.
@@ -201,6 +202,32 @@ __host__ __device__ __forceinline__ int dense_class_segments(int t, int seg_log2
     if (sh < 0) sh = 0;
     if (sh > 4) sh = 4;  // kSegGrid = 16
     return 1 << sh;
+}
+
+// Class offsets (exclusive scan of the counts) and the dense work-unit prefix,
+// by one warp.
+__device__ __forceinline__ void class_offsets(DevCounters* cnt, int seg_log2) {
+    const int lane = lane_id();
+    if (lane == 0) cnt->seg_log2 = seg_log2;
+    static_assert(kNumClasses <= 64 && kMaxDenseClasses < 32, "two classes, one dense class per lane");
+    unsigned long long base = 0;
+    for (int c0 = 0; c0 < kNumClasses; c0 += 32) {
+        const int c = c0 + lane;
+        const unsigned long long n = c < kNumClasses ? __ldcg(&cnt->class_count[c]) : 0ull;
+        const unsigned long long incl = warp_incl_scan(n);
+        if (c < kNumClasses) {
+            cnt->class_cursor[c] = base + incl - n;
+            cnt->class_off[c] = base + incl - n;
+        }
+        base += __shfl_sync(kFull, incl, 31);
+    }
+    if (lane == 0) cnt->class_off[kNumClasses] = base;
+    const unsigned long long u =
+        lane < kMaxDenseClasses
+            ? __ldcg(&cnt->class_count[kClassDense0 + lane]) * dense_class_segments(lane, seg_log2)
+            : 0ull;
+    const unsigned long long incl = warp_incl_scan(u);
+    if (lane <= kMaxDenseClasses) cnt->unit_begin[lane] = incl - u;
 }
 
 __device__ __forceinline__ long long row_end(const int64_t* rp, const int64_t* re, long long i) {
@@ -389,15 +416,23 @@ __device__ __forceinline__ void analyze_kernel_body(long long R, const ProdDesc*
     }
 }
 
+// The last block to finish also forms the class offsets.
 template <class IT, bool PREDICT>
 __global__ void __launch_bounds__(256) analyze_kernel(long long R, const ProdDesc* __restrict__ D,
                                const long long* __restrict__ rb, int nprod, long long max_dense_n,
                                int dense_min, int64_t* __restrict__ flops_out,
                                unsigned char* __restrict__ cls_out, DevCounters* cnt,
                                const float* __restrict__ prm, float margin,
-                               int64_t* __restrict__ cap_out, int hash_shift, int tile_rows) {
+                               int64_t* __restrict__ cap_out, int hash_shift, int tile_rows,
+                               int seg_log2) {
     analyze_kernel_body<IT, PREDICT>(R, D, rb, nprod, max_dense_n, dense_min, flops_out, cls_out, cnt,
         prm, margin, cap_out, hash_shift, tile_rows, (long long)blockIdx.x, (long long)gridDim.x);
+    __shared__ bool last;
+    __threadfence();   // this thread's counts come before the block's ticket
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&cnt->blocks_done, 1u) + 1u == gridDim.x;
+    __syncthreads();
+    if (last && threadIdx.x < 32) class_offsets(cnt, seg_log2);
 }
 
 // Features of every global row for the row-size predictor (log2(1 + .) of

@@ -61,7 +61,7 @@ cudaError_t launch_analyze(Plan& P) {
     count_launches(1);
     k<<<(unsigned)g, 256, 0, P.stream>>>(P.R, P.d_descs, P.rb, P.nprod, P.max_dense_n,
                                            P.dense_min, P.flops, P.cls, P.cnt, P.prm, P.margin,
-                                           P.cap, P.hash_shift, tile_rows);
+                                           P.cap, P.hash_shift, tile_rows, P.seg_log2);
     return cudaGetLastError();
 }
 
@@ -185,7 +185,8 @@ cudaError_t launch_dense_tables(Plan& P, unsigned char* ws) {
 template <class IT>
 cudaError_t launch_symbolic(Plan& P, unsigned char* ws, int64_t* rowcnt) {
     WsLayout L = workspace_layout(P);
-    cudaError_t e = launch_zero_rows(P, rowcnt);
+    // empty rows and the place of the total keep this zero
+    cudaError_t e = cudaMemsetAsync(rowcnt, 0, (size_t)(P.R + 1) * sizeof(int64_t), P.stream);
     if (e != cudaSuccess) return e;
     if ((e = sym_hash_bin<IT, 6, 8>(P, 0, rowcnt)) != cudaSuccess) return e;
     if ((e = sym_hash_bin<IT, 8, 8>(P, 1, rowcnt)) != cudaSuccess) return e;

@@ -115,7 +115,6 @@ size_t scan_temp_bytes(long long N);
 cudaError_t launch_exclusive_scan(int64_t* x, long long N, int64_t* temp, cudaStream_t s);
 cudaError_t launch_binning(Plan& P);
 cudaError_t launch_class_offsets(Plan& P);
-cudaError_t launch_zero_rows(const Plan& P, int64_t* rowcnt);
 cudaError_t launch_product_rowptr(const Plan& P, const int64_t* g, int64_t* out);
 
 // Template launchers (instantiated per index type / value type).

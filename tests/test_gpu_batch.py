@@ -298,3 +298,20 @@ def test_split3d_on_one_rank(sg, tmp_path):
         assert bool((val == C.val).all())
     finally:
         dist.destroy_process_group()
+
+
+@pytest.mark.parametrize("n", [1, 4094, 4095, 4096, 8191, 2048 * 4096 - 2, 2048 * 4096 - 1,
+                               2048 * 4096, 9_000_000])
+def test_row_pointer_scan_sizes(sg, n):
+    # the scan behind row pointers (n + 1 entries): one tile of 4096, several,
+    # and more than the 2048 tiles up to which every block adds the sums itself
+    rng = np.random.default_rng(n % 997)
+    cols = np.unique(np.concatenate([[0, n - 1], rng.integers(0, n, 5000)]))
+    reps = 1 + cols % 3
+    rows = np.concatenate([np.arange(k) for k in reps])
+    A = inputs.coo_to_csr(3, n, rows, np.repeat(cols, reps), rng.random(rows.size), np.int64)
+    T = sg.transpose(sg.to_device(A))
+    rp, col, val = T.to_host()
+    R = oracle.transpose(A)
+    assert np.array_equal(rp, R.rowptr) and np.array_equal(col, R.col)
+    assert np.array_equal(val, R.val)
