@@ -141,6 +141,16 @@ size_t plan_workspace_bytes(int nprod, long long R) {
 
 namespace sg {
 
+// The products' column chunks for the plan's chunk width.
+static void set_chunks(Plan& P) {
+    P.chunk_total = 0;
+    for (ProdDesc& d : P.descs) {
+        d.P = (int)std::max<long long>(1, (d.n + (1LL << P.cw_log2) - 1) >> P.cw_log2);
+        d.chunk_base = P.chunk_total;
+        P.chunk_total += d.m * d.P;
+    }
+}
+
 // Checks and records a batch of products; shared by spgemm_plan,
 // spgemm_batch_plan and spgemm_plan_device.
 spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
@@ -227,10 +237,12 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
         if (o.dense_chunk == sg::kDenseW0) cfg = 0;
         if (o.dense_chunk == sg::kDenseW1) cfg = 1;
         P->W = cfg == 0 ? sg::kDenseW0 : sg::kDenseW1;
+        P->cw_log2 = cfg == 0 ? 10 : 11;
     }
     P->descs.resize(count);
     std::vector<long long> rb(count + 1), bb(count + 1);
-    long long rbase = 0, bbase = 0, chunk = 0, seg = 0, run = 0;
+    long long rbase = 0, bbase = 0, seg = 0, run = 0;
+    static_assert(sg::kDenseW0 == 1 << 10 && sg::kDenseW1 == 1 << 11, "cw_log2 of both widths");
     for (int p = 0; p < count; ++p) {
         sg::ProdDesc& d = P->descs[p];
         d = sg::ProdDesc{};
@@ -247,15 +259,12 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
         d.ciB = B[p].col;
         d.vB = need_vals ? B[p].val : nullptr;
         d.nnzB = B[p].nnz;
-        d.P = (int)std::max<long long>(1, (d.n + P->W - 1) / P->W);
-        d.chunk_base = chunk;
         d.seg_base = seg;
         d.run_base = run;
         rb[p] = rbase;
         bb[p] = bbase;
         rbase += d.m;
         bbase += d.l;
-        chunk += d.m * d.P;
         seg += d.l * (sg::kSegGrid + 1);
         run += d.nnzB;
         P->max_n = std::max(P->max_n, d.n);
@@ -264,7 +273,7 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
     rb[count] = rbase;
     bb[count] = bbase;
     P->LB = bbase;
-    P->chunk_total = chunk;
+    set_chunks(*P);
     P->seg_total = seg;
     P->run_total = run;
     // plan workspace layout
@@ -369,7 +378,24 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
         // products: few, long units on big products, enough of them on small
         const double warps = (double)std::max<long long>(1, P->dense_grid * P->dense_warps_per_block);
         const double per = (double)std::max<long long>(1, P->total_flops) / (4.0 * warps);
-        P->seg_log2 = std::min(20, std::max(14, (int)std::floor(std::log2(per))));
+        P->seg_log2 = std::min(20, std::max(11, (int)std::floor(std::log2(per))));
+        // narrower chunks (16 over the widest product, at least 128 columns)
+        // where the longest row, cut into whole chunks, would still be more
+        // than a unit: a row of 18067 products in 1000 columns was one warp's
+        // work for 268 us of a 0.56 ms product (now 0.32 ms); R-MAT, 3000 vertices 0.69
+        // -> 0.45 ms, 10007 1.26 -> 0.90 ms (32 chunks: 0.50 and 0.90)
+        const long long chunks = (P->max_n + (1LL << P->cw_log2) - 1) >> P->cw_log2;
+        if (!o.dense_chunk && chunks < 16 && P->max_flops > chunks << P->seg_log2) {
+            int lg = 7;
+            while (lg < P->cw_log2 && (16LL << lg) < P->max_n) ++lg;
+            if (lg < P->cw_log2) {
+                P->cw_log2 = lg;
+                set_chunks(*P);
+                e = cudaMemcpyAsync(P->d_descs, P->descs.data(), count * sizeof(sg::ProdDesc),
+                                    cudaMemcpyHostToDevice, s);
+                if (e != cudaSuccess) return bail(cuda_fail(e, "plan: descriptor upload"));
+            }
+        }
         if (P->seg_log2 != 16) {
             e = sg::launch_class_offsets(*P);
             if (e != cudaSuccess) return bail(cuda_fail(e, "plan: work units"));
@@ -480,7 +506,7 @@ spgemm_status spgemm_plan_info(spgemm_plan_t P, spgemm_info* info) {
     for (int b = 0; b < sg::kNumHashBins; ++b) h += (long long)P->class_count[sg::kClassHash0 + b];
     info->rows_hash = h;
     info->rows_dense = P->ndense;
-    info->chunk_width = P->W;
+    info->chunk_width = 1LL << P->cw_log2;
     info->chunks_per_row = P->nprod == 1 ? P->descs[0].P : 0;
     info->nnz_c = P->nnz_c;
     return SPGEMM_OK;

@@ -116,6 +116,7 @@ spgemm_status spgemm_chain_create(int32_t nsteps, const spgemm_chain_step* steps
         c.LB = P->LB;
         c.nprod = P->nprod;
         c.W = P->W;
+        c.cw_log2 = P->cw_log2;
         c.dense_min = P->dense_min;
         c.hash_shift = P->hash_shift;
         c.seg_log2 = P->seg_log2;

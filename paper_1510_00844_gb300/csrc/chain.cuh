@@ -257,12 +257,12 @@ __global__ void __launch_bounds__(THREADS, 1)
         chain_sym_bin<IT, K, 10, BW>(c, err, bid, nb);
         chain_sym_bin<IT, K, 11, BW>(c, err, bid, nb);
         if (c.LB > 0) {
-            segtab_kernel_body<IT>(c.LB, c.D, c.bb, c.nprod, c.W, c.segtab, c.cnt, bid, nb);
-            runlen_kernel_body<IT>(c.LB, c.D, c.bb, c.nprod, c.W, c.runlen, c.nextrun, c.cnt, bid,
+            segtab_kernel_body<IT>(c.LB, c.D, c.bb, c.nprod, c.cw_log2, c.segtab, c.cnt, bid, nb);
+            runlen_kernel_body<IT>(c.LB, c.D, c.bb, c.nprod, c.cw_log2, c.runlen, c.nextrun, c.cnt, bid,
                                    nb);
         }
         symbolic_dense_kernel_body<IT, THREADS, 1>(
-            c.D, c.rb, c.nprod, c.rows, c.cnt, c.max_words, c.W / 32, c.chunkcnt, c.rowptrC,
+            c.D, c.rb, c.nprod, c.rows, c.cnt, c.max_words, 1 << (c.cw_log2 - 5), c.chunkcnt, c.rowptrC,
             &c.cnt->work_counter[0], err, bid, nb, sym_groups);
         if (!chain_barrier(sync, stage++)) return;
         // row pointers: exclusive scan of the counts (R + 1 entries)
@@ -282,12 +282,14 @@ __global__ void __launch_bounds__(THREADS, 1)
                 numeric_dense_kernel_body<IT, V, kDenseW0, kChainDense0>(
                 c.D, c.rb, c.nprod, c.rows, c.cnt, c.chunkcnt, c.segtab, c.runlen, c.nextrun,
                 c.arena, c.arena_stride, c.rowptrC, c.capacity, colC, valC, c.max_dense_n,
-                &c.cnt->work_counter[1], err, nullptr, nullptr, nullptr, nullptr, bid, nb);
+                &c.cnt->work_counter[1], err, nullptr, nullptr, nullptr, nullptr, c.cw_log2, bid,
+                nb);
         } else if (threadIdx.x < kChainDense1 * 32) {
             numeric_dense_kernel_body<IT, V, kDenseW1, kChainDense1>(
                 c.D, c.rb, c.nprod, c.rows, c.cnt, c.chunkcnt, c.segtab, c.runlen, c.nextrun,
                 c.arena, c.arena_stride, c.rowptrC, c.capacity, colC, valC, c.max_dense_n,
-                &c.cnt->work_counter[1], err, nullptr, nullptr, nullptr, nullptr, bid, nb);
+                &c.cnt->work_counter[1], err, nullptr, nullptr, nullptr, nullptr, c.cw_log2, bid,
+                nb);
         }
         if (!chain_barrier(sync, stage++)) return;
     }

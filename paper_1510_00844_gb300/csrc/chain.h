@@ -40,7 +40,7 @@ struct ChainProduct {
     void* colC;
     void* valC;
     long long R, LB, max_dense_n, arena_stride, capacity;
-    int nprod, W, dense_min, hash_shift, seg_log2, max_words;
+    int nprod, W, cw_log2, dense_min, hash_shift, seg_log2, max_words;
 };
 
 // Barrier state (first 16 bytes cleared by the host before every launch)

@@ -1771,7 +1771,8 @@ __global__ void __launch_bounds__(32 * kRankWarps)
 }
 
 // --------------------------------------------------- numeric: dense rows
-// Work units: a dense row's P column chunks (width W) are cut into G equal
+// Work units: a dense row's P column chunks (of 2^cw_log2 <= W columns: W
+// unless the plan needs more units than that leaves) are cut into G equal
 // segments (G in {1, 2, 4, ..., kSegGrid}, chosen per flops class so that a
 // unit carries a bounded share of flops); one warp owns a unit.  For each
 // chunk of its segment the warp walks A(i,:) in order and, per entry, the part
@@ -1796,7 +1797,7 @@ struct __align__(16) DenseCursor {
 };
 
 // runlen[run_base + q] = number of entries from q to the end of q's column
-// chunk (col / W) inside its row of B: the length of the part of B(k,:) that
+// chunk (col >> cw_log2) inside its row of B: the length of the part of B(k,:) that
 // a chunk sweep consumes in one step.  nextrun[run_base + q] = {length, first
 // column} of the run that follows the one starting at q ({0, INT_MAX} at the
 // row's end), so a cursor advances with one load whose address it knows
@@ -1805,7 +1806,7 @@ struct __align__(16) DenseCursor {
 // successor table in a forward pass over what the warp wrote.
 template <class IT>
 __device__ __forceinline__ void runlen_kernel_body(long long LB, const ProdDesc* __restrict__ D,
-                              const long long* __restrict__ bb, int nprod, int W,
+                              const long long* __restrict__ bb, int nprod, int cw_log2,
                               int32_t* __restrict__ runlen, int2* __restrict__ nextrun,
                               const DevCounters* cnt,
         const long long vbid, const long long vnb) {
@@ -1827,7 +1828,7 @@ __device__ __forceinline__ void runlen_kernel_body(long long LB, const ProdDesc*
             const long long lo = max(s0, hi - 32);
             const long long q = lo + lane;
             const bool in = q < hi;
-            const long long ch = in ? (long long)ciB[q] / W : -2;
+            const long long ch = in ? (long long)ciB[q] >> cw_log2 : -2;
             long long nxt = __shfl_down_sync(kFull, ch, 1);
             if (lane == 31 || q + 1 >= hi) nxt = carry_chunk;
             const bool last = in && nxt != ch;   // q ends its run inside this window
@@ -1854,18 +1855,18 @@ __device__ __forceinline__ void runlen_kernel_body(long long LB, const ProdDesc*
 
 template <class IT>
 __global__ void runlen_kernel(long long LB, const ProdDesc* __restrict__ D,
-                              const long long* __restrict__ bb, int nprod, int W,
+                              const long long* __restrict__ bb, int nprod, int cw_log2,
                               int32_t* __restrict__ runlen, int2* __restrict__ nextrun,
                               const DevCounters* cnt) {
-    runlen_kernel_body<IT>(LB, D, bb, nprod, W, runlen, nextrun, cnt, (long long)blockIdx.x,
+    runlen_kernel_body<IT>(LB, D, bb, nprod, cw_log2, runlen, nextrun, cnt, (long long)blockIdx.x,
         (long long)gridDim.x);
 }
 
 // segtab[seg_base + k * (kSegGrid+1) + g] = first position p in B(k,:) with
-// col >= seg_chunk(g, P) * W, relative to rowptr[k].
+// col >= seg_chunk(g, P) << cw_log2, relative to rowptr[k].
 template <class IT>
 __device__ __forceinline__ void segtab_kernel_body(long long LB, const ProdDesc* __restrict__ D,
-                              const long long* __restrict__ bb, int nprod, int W,
+                              const long long* __restrict__ bb, int nprod, int cw_log2,
                               int32_t* __restrict__ segtab, const DevCounters* cnt,
         const long long vbid, const long long vnb) {
     if (cnt->class_off[kNumClasses] == cnt->class_off[kClassDense0]) return;  // no dense rows
@@ -1878,7 +1879,7 @@ __device__ __forceinline__ void segtab_kernel_body(long long LB, const ProdDesc*
         const ProdDesc& d = D[pr];
         const long long k = kb - d.brow_base;
         const IT* ciB = (const IT*)d.ciB;
-        const long long key = seg_chunk(g, d.P) * W;
+        const long long key = seg_chunk(g, d.P) << cw_log2;
         long long lo = d.rpB[k], hi = d.rpB[k + 1];
         const long long base = lo;
         while (lo < hi) {
@@ -1892,9 +1893,9 @@ __device__ __forceinline__ void segtab_kernel_body(long long LB, const ProdDesc*
 
 template <class IT>
 __global__ void segtab_kernel(long long LB, const ProdDesc* __restrict__ D,
-                              const long long* __restrict__ bb, int nprod, int W,
+                              const long long* __restrict__ bb, int nprod, int cw_log2,
                               int32_t* __restrict__ segtab, const DevCounters* cnt) {
-    segtab_kernel_body<IT>(LB, D, bb, nprod, W, segtab, cnt, (long long)blockIdx.x,
+    segtab_kernel_body<IT>(LB, D, bb, nprod, cw_log2, segtab, cnt, (long long)blockIdx.x,
         (long long)gridDim.x);
 }
 
@@ -1990,7 +1991,7 @@ __device__ __forceinline__ void numeric_dense_kernel_body(
                          V* __restrict__ vC, long long max_dense_n, unsigned long long* work,
                          int* err, int64_t* __restrict__ rowend, int32_t* __restrict__ overflow,
                          unsigned* overflow_count, int64_t* __restrict__ unit_cnt,
-        const long long vbid, const long long vnb) {
+        const int cw_log2, const long long vbid, const long long vnb) {
     constexpr bool HV = VOps<V>::has_val;
     constexpr int kNone = 0x7fffffff;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -2088,9 +2089,9 @@ __device__ __forceinline__ void numeric_dense_kernel_body(
         }
         min_next = warp_min(min_next);
         __syncwarp();
-        for (int c = max(cs, min_next / W); c < ce;) {
-            const long long c0 = (long long)c * W;
-            const long long c1 = min(c0 + (long long)W, n);
+        for (int c = max(cs, min_next >> cw_log2); c < ce;) {
+            const long long c0 = (long long)c << cw_log2;
+            const long long c1 = min(c0 + (1LL << cw_log2), n);
             int cnext = kNone;  // smallest column after this chunk
             // batches of 32 entries: cursors and A values are loaded together
             // (neither address depends on the other); a cursor's next run is
@@ -2122,10 +2123,10 @@ __device__ __forceinline__ void numeric_dense_kernel_body(
             // emit the chunk in column order: lane t owns bitmap word t (32
             // columns), a warp scan of the popcounts gives each lane its output
             // run; words and values are reset on the way
-            constexpr int NWORDS = W / 32;
-            for (int t0 = 0; t0 < NWORDS; t0 += 32) {
+            const int nwords = 1 << (cw_log2 - 5);
+            for (int t0 = 0; t0 < nwords; t0 += 32) {
                 const int wi0 = t0 + lane;
-                unsigned word = wi0 < NWORDS ? bm[wi0] : 0u;
+                unsigned word = wi0 < nwords ? bm[wi0] : 0u;
                 const int pc = __popc(word);
                 const int pincl = warp_incl_scan(pc);
                 long long pos = out + (pincl - pc);
@@ -2140,11 +2141,11 @@ __device__ __forceinline__ void numeric_dense_kernel_body(
                     if constexpr (HV) acc[s] = VOps<V>::init();
                     ++pos;
                 }
-                if (wi0 < NWORDS) bm[wi0] = 0u;
+                if (wi0 < nwords) bm[wi0] = 0u;
                 out += __shfl_sync(kFull, pincl, 31);
             }
             __syncwarp();
-            const int jump = warp_min(cnext) / W;
+            const int jump = warp_min(cnext) >> cw_log2;
             c = max(c + 1, jump);
         }
         if (lane == 0) {
@@ -2170,10 +2171,10 @@ __global__ void __launch_bounds__(WARPS * 32, 24 / WARPS)
                          const int64_t* __restrict__ rpC, long long cap, IT* __restrict__ ciC,
                          V* __restrict__ vC, long long max_dense_n, unsigned long long* work,
                          int* err, int64_t* __restrict__ rowend, int32_t* __restrict__ overflow,
-                         unsigned* overflow_count, int64_t* __restrict__ unit_cnt) {
+                         unsigned* overflow_count, int64_t* __restrict__ unit_cnt, int cw_log2) {
     numeric_dense_kernel_body<IT, V, W, WARPS>(D, rb, nprod, rows, cnt, chunkcnt, segtab, runlen,
         nextrun, arena, arena_stride, rpC, cap, ciC, vC, max_dense_n, work, err, rowend,
-        overflow, overflow_count, unit_cnt, (long long)blockIdx.x, (long long)gridDim.x);
+        overflow, overflow_count, unit_cnt, cw_log2, (long long)blockIdx.x, (long long)gridDim.x);
 }
 
 // Learned sizing: close the gaps a slot-mode dense row leaves between its

@@ -169,12 +169,12 @@ cudaError_t launch_dense_tables(Plan& P, unsigned char* ws) {
         long long total = P.LB * (kSegGrid + 1);
         long long g = grid_for(total, 256, P.sm_count, 8);
         count_launches(1);
-        segtab_kernel<IT><<<(unsigned)g, 256, 0, P.stream>>>(P.LB, P.d_descs, P.bb, P.nprod, P.W,
+        segtab_kernel<IT><<<(unsigned)g, 256, 0, P.stream>>>(P.LB, P.d_descs, P.bb, P.nprod, P.cw_log2,
                                                              (int32_t*)(ws + L.segtab), P.cnt);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         long long g2 = grid_for(P.LB, 8, P.sm_count, 8);
         count_launches(1);
-        runlen_kernel<IT><<<(unsigned)g2, 256, 0, P.stream>>>(P.LB, P.d_descs, P.bb, P.nprod, P.W,
+        runlen_kernel<IT><<<(unsigned)g2, 256, 0, P.stream>>>(P.LB, P.d_descs, P.bb, P.nprod, P.cw_log2,
                                                               (int32_t*)(ws + L.runlen),
                                                               (int2*)(ws + L.nextrun), P.cnt);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -216,12 +216,12 @@ cudaError_t launch_symbolic(Plan& P, unsigned char* ws, int64_t* rowcnt) {
         count_launches(1);
         if (threads == 1024)
             kb<<<(unsigned)g, threads, smem, P.stream>>>(P.d_descs, P.rb, P.nprod, P.rows, P.cnt,
-                                                         max_words, P.W / 32,
+                                                         max_words, 1 << (P.cw_log2 - 5),
                                                          (int32_t*)(ws + L.chunkcnt), rowcnt, work,
                                                          &P.cnt->err);
         else
             ks<<<(unsigned)g, threads, smem, P.stream>>>(P.d_descs, P.rb, P.nprod, P.rows, P.cnt,
-                                                         max_words, P.W / 32,
+                                                         max_words, 1 << (P.cw_log2 - 5),
                                                          (int32_t*)(ws + L.chunkcnt), rowcnt, work,
                                                          &P.cnt->err);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -274,7 +274,7 @@ cudaError_t launch_numeric_dense(Plan& P, unsigned char* ws, const int64_t* rpC,
         P.d_descs, P.rb, P.nprod, P.rows, P.cnt, (const int32_t*)(ws + L.chunkcnt),
         (const int32_t*)(ws + L.segtab), (const int32_t*)(ws + L.runlen),
         (const int2*)(ws + L.nextrun), (DenseCursor*)(ws + L.arena), L.arena_stride, rpC, cap, colC, valC, P.max_dense_n, work,
-        &P.cnt->err, rowend, overflow, overflow_count, P.unit_cnt);
+        &P.cnt->err, rowend, overflow, overflow_count, P.unit_cnt, P.cw_log2);
     return cudaGetLastError();
 }
 

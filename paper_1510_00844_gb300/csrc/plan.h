@@ -50,7 +50,8 @@ struct spgemm_plan_s {
     long long class_off[sg::kNumClasses + 1] = {};
     long long total_flops = 0, max_flops = 0;
     long long ndense = 0;
-    int W = 1024;            // dense chunk width (columns)
+    int W = 1024;            // accumulators of a dense chunk (columns)
+    int cw_log2 = 10;        // dense chunk width: at most W
     long long max_dense_len = 0;  // cursor arena slot (entries)
     long long dense_grid = 0;     // blocks of the dense numeric kernel
     int dense_warps_per_block = 8;

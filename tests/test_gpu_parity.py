@@ -535,3 +535,28 @@ def test_rows_of_129_to_1024_products(sg, n, value):
         assert_values_close(C, R, A, B, "f32")
     elif value != "none":
         assert np.array_equal(C.to_host()[2], R.val)
+
+
+@pytest.mark.parametrize("n,l,value", [(130, 300, "u01_f64"), (700, 200, "none"),
+                                       (1025, 150, "u11_f32"), (2047, 120, "int"),
+                                       (3001, 100, "u01_f64"), (16500, 60, "u01_f64")])
+def test_dense_rows_in_narrow_chunks(sg, n, l, value):
+    """Few columns, long rows: the chunks of the dense rows are narrowed (down to
+    128 columns) so that a row makes several work units; 16500 columns keep
+    the full width for float64.  Plain and learned sizing."""
+    A = inputs.random_csr(90, l, 0.6, 31 + n, value=value, index_dtype=np.int32)
+    B = inputs.random_csr(l, n, 0.5, 32 + n, value=value, index_dtype=np.int32, empty_rows=0.1)
+    sr = 1 if value == "none" else 0
+    C = run(sg, A, B, semiring=sr)
+    R = oracle.spgemm(A, B, semiring="or_and" if sr else "plus_times")
+    assert_pattern_equal(C, R)
+    if value == "u11_f32":
+        assert_values_close(C, R, A, B, "f32")
+    elif value != "none":
+        assert np.array_equal(C.to_host()[2], R.val)
+    L, _ = sg.learned_multiply(sg.to_device(A), sg.to_device(B), sg.sizer_init(seed=3), 0.2,
+                               semiring=sr)
+    L = sg.compact(L) if L.rowend is not None else L
+    assert bool((L.col == C.col).all()) and bool((L.rowptr == C.rowptr).all())
+    if value != "none":
+        assert bool((L.val == C.val).all())
