@@ -18,6 +18,7 @@
 #pragma once
 
 #include "device_common.cuh"
+#include "rows.cuh"
 
 namespace sg {
 
@@ -1796,14 +1797,95 @@ struct __align__(16) DenseCursor {
     int rl;
 };
 
-// runlen[run_base + q] = number of entries from q to the end of q's column
-// chunk (col >> cw_log2) inside its row of B: the length of the part of B(k,:) that
-// a chunk sweep consumes in one step.  nextrun[run_base + q] = {length, first
-// column} of the run that follows the one starting at q ({0, INT_MAX} at the
-// row's end), so a cursor advances with one load whose address it knows
-// before the chunk's products are accumulated.  One warp per B row of every
-// product: run lengths in windows of 32 from the row end backwards, then the
-// successor table in a forward pass over what the warp wrote.
+// Run tables of B, at the positions where a run (the entries of B(k,:) inside
+// one column chunk, col >> cw_log2) starts: runlen[run_base + q] = its length,
+// nextrun[run_base + q] = {length, first column} of the run after it ({0,
+// INT_MAX} at the row's end), so a cursor advances with one load whose address
+// it knows before the chunk's products are accumulated.  Other positions are not
+// written: a cursor only ever stands at the start of a run.  Warp w of WARPS
+// takes every WARPS-th window of 32 entries of the row; the run that leaves a
+// window is followed by a search.  (With a warp per row, window after window
+// from the row's end, and both tables at every entry, the longest rows alone
+// took most of the 613 us of an R-MAT 18 square; now 218 us.)
+template <class IT, int WARPS>
+__device__ __forceinline__ void run_tables_row(const IT* __restrict__ ci, long long s0,
+                                               long long s1, int cw_log2, int32_t* rl, int2* nr,
+                                               int w) {
+    const int lane = lane_id();
+    if (WARPS == 1 && s1 - s0 <= 32) {   // one window: the next run is a lane of it
+        const long long q = s0 + lane;
+        const int col = q < s1 ? (int)ci[q] : 0x7fffffff;
+        const int before = __shfl_up_sync(kFull, col, 1);
+        const bool start = q < s1 && (lane == 0 || before >> cw_log2 != col >> cw_log2);
+        const unsigned later = __ballot_sync(kFull, start) & ~lanemask_le();
+        const int next = later ? __ffs(later) - 1 : (int)(s1 - s0);
+        const int len = next - lane;
+        const int next_len = __shfl_sync(kFull, len, next & 31);
+        const int next_col = __shfl_sync(kFull, col, next & 31);
+        if (start) {
+            rl[q] = len;
+            nr[q] = later ? make_int2(next_len, next_col) : make_int2(0, 0x7fffffff);
+        }
+        return;
+    }
+    // whether q starts a run, from its chunk and the chunk of the entry before it
+    auto starts = [&](long long q, long long& ch) {
+        ch = q < s1 ? (long long)ci[q] >> cw_log2 : -2;
+        long long before = __shfl_up_sync(kFull, ch, 1);
+        if (lane == 0) before = q > s0 && q < s1 ? (long long)ci[q - 1] >> cw_log2 : -1;
+        return q < s1 && before != ch;
+    };
+    for (long long lo = s0 + 32 * w; lo < s1; lo += 32 * WARPS) {
+        const long long q = lo + lane;
+        long long ch;
+        const bool start = starts(q, ch);
+        const unsigned later = __ballot_sync(kFull, start) & ~lanemask_le();
+        if (start) {
+            long long end = q + __ffs(later) - 1 - lane;   // the next start in the window
+            if (later == 0u) {
+                // first entry past the window in another chunk; a run has at
+                // most 2^cw_log2 entries
+                long long p = min(s1, lo + 32), e = min(s1, q + (1LL << cw_log2));
+                if (p < e && (long long)ci[p] >> cw_log2 != ch) e = p;
+                while (p < e) {
+                    const long long mid = (p + e) >> 1;
+                    if ((long long)ci[mid] >> cw_log2 == ch) p = mid + 1;
+                    else e = mid;
+                }
+                end = p;
+            }
+            rl[q] = (int32_t)(end - q);
+        }
+    }
+    if constexpr (WARPS > 1) __syncthreads();   // the row's run lengths are visible
+    else __syncwarp();
+    for (long long lo = s0 + 32 * w; lo < s1; lo += 32 * WARPS) {
+        const long long q = lo + lane;
+        long long ch;
+        if (starts(q, ch)) {
+            const long long q2 = q + rl[q];
+            nr[q] = q2 < s1 ? make_int2(rl[q2], (int)ci[q2]) : make_int2(0, 0x7fffffff);
+        }
+    }
+    __syncwarp();
+}
+
+template <class IT>
+struct BRow {
+    const IT* ci;
+    long long s0, s1, run_base;
+};
+
+template <class IT>
+__device__ __forceinline__ BRow<IT> b_row(const ProdDesc* __restrict__ D,
+                                          const long long* __restrict__ bb, int nprod,
+                                          long long kb) {
+    const ProdDesc& d = D[nprod > 1 ? find_prod(bb, nprod, kb) : 0];
+    const long long k = kb - d.brow_base;
+    return BRow<IT>{(const IT*)d.ciB, d.rpB[k], d.rpB[k + 1], d.run_base};
+}
+
+// A warp per B row (inside the persistent chain).
 template <class IT>
 __device__ __forceinline__ void runlen_kernel_body(long long LB, const ProdDesc* __restrict__ D,
                               const long long* __restrict__ bb, int nprod, int cw_log2,
@@ -1811,55 +1893,44 @@ __device__ __forceinline__ void runlen_kernel_body(long long LB, const ProdDesc*
                               const DevCounters* cnt,
         const long long vbid, const long long vnb) {
     if (cnt->class_off[kNumClasses] == cnt->class_off[kClassDense0]) return;  // no dense rows
-    const int lane = lane_id();
     const long long warp = ((long long)vbid * blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)vnb * blockDim.x) >> 5;
     for (long long kb = warp; kb < LB; kb += nwarps) {
-        const int pr = nprod > 1 ? find_prod(bb, nprod, kb) : 0;
-        const ProdDesc& d = D[pr];
-        const long long k = kb - d.brow_base;
-        const IT* ciB = (const IT*)d.ciB;
-        int32_t* rl = runlen + d.run_base;
-        int2* nr = nextrun + d.run_base;
-        const long long s0 = d.rpB[k], s1 = d.rpB[k + 1];
-        long long carry_end = s1;          // run end of the window after this one
-        long long carry_chunk = -1;        // chunk of the first entry of that window
-        for (long long hi = s1; hi > s0; hi -= 32) {
-            const long long lo = max(s0, hi - 32);
-            const long long q = lo + lane;
-            const bool in = q < hi;
-            const long long ch = in ? (long long)ciB[q] >> cw_log2 : -2;
-            long long nxt = __shfl_down_sync(kFull, ch, 1);
-            if (lane == 31 || q + 1 >= hi) nxt = carry_chunk;
-            const bool last = in && nxt != ch;   // q ends its run inside this window
-            const unsigned lm = __ballot_sync(kFull, last);
-            const unsigned ge = lm & (0xffffffffu << lane);
-            long long end;
-            if (ge) end = lo + (__ffs(ge) - 1) + 1;
-            else end = carry_end;
-            if (in) rl[q] = (int32_t)(end - q);
-            // first entry of this window seeds the carry for the window before it
-            carry_end = __shfl_sync(kFull, end, 0);
-            carry_chunk = __shfl_sync(kFull, ch, 0);
-        }
-        __syncwarp();   // the run lengths of the whole row are visible to the warp
-        for (long long q = s0 + lane; q < s1; q += 32) {
-            const long long q2 = q + rl[q];
-            int2 x = make_int2(0, 0x7fffffff);
-            if (q2 < s1) x = make_int2(rl[q2], (int)ciB[q2]);
-            nr[q] = x;
-        }
-        __syncwarp();
+        const BRow<IT> r = b_row<IT>(D, bb, nprod, kb);
+        run_tables_row<IT, 1>(r.ci, r.s0, r.s1, cw_log2, runlen + r.run_base,
+                              nextrun + r.run_base, 0);
     }
 }
 
+// A warp per B row, a block for the longest.
 template <class IT>
-__global__ void runlen_kernel(long long LB, const ProdDesc* __restrict__ D,
-                              const long long* __restrict__ bb, int nprod, int cw_log2,
-                              int32_t* __restrict__ runlen, int2* __restrict__ nextrun,
-                              const DevCounters* cnt) {
-    runlen_kernel_body<IT>(LB, D, bb, nprod, cw_log2, runlen, nextrun, cnt, (long long)blockIdx.x,
-        (long long)gridDim.x);
+__global__ void __launch_bounds__(32 * kRowWarps)
+    runlen_kernel(long long LB, const ProdDesc* __restrict__ D,
+                  const long long* __restrict__ bb, int nprod, int cw_log2,
+                  int32_t* __restrict__ runlen, int2* __restrict__ nextrun,
+                  const DevCounters* cnt) {
+    if (cnt->class_off[kNumClasses] == cnt->class_off[kClassDense0]) return;  // no dense rows
+    // as for_rows, but a row of a batch is looked up once
+    __shared__ BRow<IT> longs[kRowWarps];
+    const int w = threadIdx.x >> 5;
+    for (long long tile = blockIdx.x; tile * kRowWarps < LB; tile += gridDim.x) {
+        const long long kb = tile * kRowWarps + w;
+        BRow<IT> r{nullptr, 0, 0, 0};
+        if (kb < LB) r = b_row<IT>(D, bb, nprod, kb);
+        const bool big = r.s1 - r.s0 > 512;
+        if (!big && r.s1 > r.s0)
+            run_tables_row<IT, 1>(r.ci, r.s0, r.s1, cw_log2, runlen + r.run_base,
+                                  nextrun + r.run_base, 0);
+        if (lane_id() == 0) longs[w] = big ? r : BRow<IT>{nullptr, 0, 0, 0};
+        if (__syncthreads_or(big))
+            for (int t = 0; t < kRowWarps; ++t) {
+                const BRow<IT> x = longs[t];
+                if (x.s1 > x.s0)
+                    run_tables_row<IT, kRowWarps>(x.ci, x.s0, x.s1, cw_log2, runlen + x.run_base,
+                                                  nextrun + x.run_base, w);
+            }
+        __syncthreads();   // the list has been read
+    }
 }
 
 // segtab[seg_base + k * (kSegGrid+1) + g] = first position p in B(k,:) with
