@@ -112,15 +112,20 @@ WsLayout workspace_layout(const Plan& P) {
     size_t off = 0;
     L.chunkcnt = off;
     if (dense) off += align_up((size_t)P.chunk_total * sizeof(int32_t));
+    L.kept = off;
+    if (P.keep_bits)
+        off += align_up((size_t)P.ndense * ((std::min(P.max_n, P.max_dense_n) + 31) / 32) *
+                        sizeof(unsigned));
+    const bool tables = dense && !P.keep_bits;   // what the sweep over the products needs
     L.segtab = off;
-    if (dense) off += align_up((size_t)P.seg_total * sizeof(int32_t));
+    if (tables) off += align_up((size_t)P.seg_total * sizeof(int32_t));
     L.runlen = off;
-    if (dense) off += align_up((size_t)P.run_total * sizeof(int32_t));
+    if (tables) off += align_up((size_t)P.run_total * sizeof(int32_t));
     L.nextrun = off;
-    if (dense) off += align_up((size_t)P.run_total * sizeof(int2));
+    if (tables) off += align_up((size_t)P.run_total * sizeof(int2));
     L.arena = off;
     L.arena_stride = std::max<long long>(1, P.max_dense_len);
-    if (dense)
+    if (tables)
         off += align_up((size_t)P.dense_grid * P.dense_warps_per_block * (size_t)L.arena_stride *
                         sizeof(DenseCursor));
     L.scan = off;
@@ -373,6 +378,14 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
     P->max_dense_len = (long long)h.max_dense_len;
     e = prepare();
     if (e != cudaSuccess) return bail(cuda_fail(e, "plan: numeric setup"));
+    {
+        // A pattern's dense rows are in the bitmaps of the symbolic pass: they
+        // are kept while they take no more than a byte per product (the columns
+        // of C take up to four) and 8 GB.  Learned plans have no symbolic pass.
+        const double bytes = (double)P->ndense * (double)std::min(P->max_n, P->max_dense_n) / 8;
+        P->keep_bits = vt == SPGEMM_BOOL && !P->prm && P->ndense > 0 &&
+                       bytes <= (double)P->total_flops && bytes <= 8e9;
+    }
     if (!o.seg_log2 && P->ndense > 0) {
         // dense work units of about total_flops / (4 x resident dense warps)
         // products: few, long units on big products, enough of them on small

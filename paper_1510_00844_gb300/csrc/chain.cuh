@@ -263,7 +263,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         symbolic_dense_kernel_body<IT, THREADS, 1>(
             c.D, c.rb, c.nprod, c.rows, c.cnt, c.max_words, 1 << (c.cw_log2 - 5), c.chunkcnt, c.rowptrC,
-            &c.cnt->work_counter[0], err, bid, nb, sym_groups);
+            &c.cnt->work_counter[0], err, nullptr, bid, nb, sym_groups);
         if (!chain_barrier(sync, stage++)) return;
         // row pointers: exclusive scan of the counts (R + 1 entries)
         chain_scan_sums(c.rowptrC, c.R + 1, c.scan, bid, nb);

@@ -164,7 +164,8 @@ template <class IT>
 cudaError_t launch_dense_tables(Plan& P, unsigned char* ws) {
     WsLayout L = workspace_layout(P);
     cudaError_t e = cudaSuccess;
-    const bool dense = P.device_sized || P.ndense > 0;
+    // columns that come from kept bitmaps need no tables of B
+    const bool dense = (P.device_sized || P.ndense > 0) && !P.keep_bits;
     if (dense && P.LB > 0) {
         long long total = P.LB * (kSegGrid + 1);
         long long g = grid_for(total, 256, P.sm_count, 8);
@@ -211,6 +212,7 @@ cudaError_t launch_symbolic(Plan& P, unsigned char* ws, int64_t* rowcnt) {
         if (o1024 * 1024 > occ * threads) { threads = 1024; occ = o1024; }
         long long g = class_grid(P, P.ndense, 1, occ);
         unsigned long long* work = &P.cnt->work_counter[0];
+        unsigned* kept = P.keep_bits ? (unsigned*)(ws + L.kept) : nullptr;
         if ((e = cudaMemsetAsync(work, 0, sizeof(unsigned long long), P.stream)) != cudaSuccess)
             return e;
         count_launches(1);
@@ -218,12 +220,12 @@ cudaError_t launch_symbolic(Plan& P, unsigned char* ws, int64_t* rowcnt) {
             kb<<<(unsigned)g, threads, smem, P.stream>>>(P.d_descs, P.rb, P.nprod, P.rows, P.cnt,
                                                          max_words, 1 << (P.cw_log2 - 5),
                                                          (int32_t*)(ws + L.chunkcnt), rowcnt, work,
-                                                         &P.cnt->err);
+                                                         &P.cnt->err, kept);
         else
             ks<<<(unsigned)g, threads, smem, P.stream>>>(P.d_descs, P.rb, P.nprod, P.rows, P.cnt,
                                                          max_words, 1 << (P.cw_log2 - 5),
                                                          (int32_t*)(ws + L.chunkcnt), rowcnt, work,
-                                                         &P.cnt->err);
+                                                         &P.cnt->err, kept);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -289,6 +291,17 @@ cudaError_t launch_numeric(Plan& P, unsigned char* ws, const int64_t* rpC, long 
     if ((e = num_hash_bin<IT, V, 8, 8>(P, 1, rpC, cap, colC, valC, rowend, overflow, overflow_count)) != cudaSuccess) return e;
     if ((e = num_hash_bin<IT, V, 10, 8>(P, 2, rpC, cap, colC, valC, rowend, overflow, overflow_count)) != cudaSuccess) return e;
     if ((e = num_hash_bin<IT, V, 11, 4>(P, 3, rpC, cap, colC, valC, rowend, overflow, overflow_count)) != cudaSuccess) return e;
+    if (P.keep_bits) {
+        WsLayout L = workspace_layout(P);
+        auto k = dense_columns_kernel<IT>;
+        const int occ = occupancy_blocks(k, 256, 0);
+        count_launches(1);
+        k<<<(unsigned)grid_for(P.ndense, 1, P.sm_count, occ), 256, 0, P.stream>>>(
+            P.d_descs, P.rb, P.nprod, P.rows, P.cnt, (const unsigned*)(ws + L.kept),
+            (int)((std::min(P.max_n, P.max_dense_n) + 31) / 32), 1 << (P.cw_log2 - 5),
+            (const int32_t*)(ws + L.chunkcnt), rpC, cap, colC, &P.cnt->err);
+        return cudaGetLastError();
+    }
     if (P.device_sized || P.ndense > 0) {
         e = P.W == kDenseW0
                 ? launch_numeric_dense<IT, V, kDenseW0, kDenseWarps0>(P, ws, rpC, cap, colC, valC,

@@ -31,6 +31,7 @@ struct spgemm_plan_s {
     int hash_shift = 0;      // hash rows are binned by flops << hash_shift
     int seg_log2 = 16;       // dense work units of about 2^seg_log2 products
     bool device_sized = false;  // no host readback: sizes are upper bounds
+    bool keep_bits = false;  // pattern only: the symbolic pass keeps the dense rows' bitmaps
     // plan workspace
     unsigned char* pws = nullptr;
     size_t pws_bytes = 0;
@@ -94,7 +95,7 @@ void count_launches(long long k);
 void set_last_error(const char* msg);
 
 struct WsLayout {
-    size_t chunkcnt = 0, segtab = 0, runlen = 0, nextrun = 0, arena = 0, scan = 0, total = 0;
+    size_t chunkcnt = 0, kept = 0, segtab = 0, runlen = 0, nextrun = 0, arena = 0, scan = 0, total = 0;
     long long arena_stride = 0;
 };
 WsLayout workspace_layout(const Plan& P);

@@ -560,3 +560,31 @@ def test_dense_rows_in_narrow_chunks(sg, n, l, value):
     assert bool((L.col == C.col).all()) and bool((L.rowptr == C.rowptr).all())
     if value != "none":
         assert bool((L.val == C.val).all())
+
+
+@pytest.mark.parametrize("n,rows,l,density", [(40000, 40, 300, 0.2), (65600, 7, 40, 0.9),
+                                              (200_000, 9, 30, 0.002), (1500, 60, 80, 0.99)])
+@pytest.mark.parametrize("index", [np.int32, np.int64])
+def test_pattern_of_dense_rows(sg, n, rows, l, density, index):
+    """Dense rows of a pattern, from the bitmaps the symbolic pass keeps (all
+    cases but the third, whose bitmaps would take more bytes than there are
+    products) and, with a second numeric pass, from them again; nearly full and
+    sparse words, widths that are not whole words or chunks."""
+    rng = np.random.default_rng(n % 991)
+    A = inputs.random_csr(rows, l, 0.9, 41 + l, value="none", index_dtype=index)
+    cols = [np.flatnonzero(rng.random(n) < density) for _ in range(l)]
+    cols[0] = np.array([0, n - 1])
+    B = inputs.CSR(l, n, np.concatenate([[0], np.cumsum([c.size for c in cols])]).astype(np.int64),
+                   np.concatenate(cols).astype(index), None)
+    dA, dB = sg.to_device(A), sg.to_device(B)
+    p = sg.plan(dA, dB, semiring=1)
+    assert p.info()["rows_dense"] > 0
+    rp, nnz = sg.symbolic(p)
+    R = oracle.spgemm(A, B, semiring="or_and")
+    for _ in range(2):
+        col, val = sg.alloc_output(p, nnz)
+        col.fill_(-1)
+        sg.numeric(p, rp, col, val)
+        sg.check(p)
+        assert np.array_equal(rp.cpu().numpy(), R.rowptr)
+        assert np.array_equal(col.cpu().numpy().astype(np.int64), R.col)
