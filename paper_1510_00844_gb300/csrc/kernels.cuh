@@ -918,8 +918,9 @@ __global__ void __launch_bounds__(WARPS * 32)
 // per-chunk counts chunkcnt[chunk_base + i*P + c] (chunk c covers columns
 // [c*W, (c+1)*W)), which the numeric phase uses to skip empty chunks.
 // MAXT / MINB: launch bounds of the instantiation (a register cap that lets
-// six 256-thread or three 512-thread blocks share an SM, or one 1024-thread
-// block for a bitmap that leaves room for only one block).
+// four 256-thread or two 512-thread blocks share an SM -- for six and three it
+// spills, 0.085 against 0.074 ms on 10007 vertices -- or one 1024-thread block
+// for a bitmap that leaves room for only one block).
 // Groups: the block may be split into `groups` equal groups of whole warps
 // (named barriers 1..groups), each with its own bitmap of max_words words,
 // so that several rows are in flight in one block; groups == 1 is the
@@ -929,6 +930,88 @@ constexpr int kMaxSymGroups = 8;
 __device__ __forceinline__ void group_sync(int g, int gthreads, int groups) {
     if (groups == 1) __syncthreads();
     else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "r"(gthreads) : "memory");
+}
+
+// Sets the bits of the row's columns, by `nwarps` warps together (the order does
+// not matter).  A entries are taken 32 at a time: by all warps while the row
+// has no more than 32 per warp -- each then takes every nwarps-th piece of 256
+// products -- else by one warp each.  (One warp per 32 entries whatever the row
+// left the others waiting for it: rows of 17 A entries hold 16000 to 65000
+// products of an R-MAT 18 square, and the pass spent 16 of 26 cycles between
+// instructions at the barrier.)  Long rows of B go eight loads at a time.  One
+// shared atomic per product: OR-ing the lanes' bits of a common word first (a
+// segmented scan, or __match_any_sync with __reduce_or_sync) was measured 3x and
+// 5x slower, testing the bit before 1.3x.
+// R-MAT 18: 11.9 -> 7.2 ms; 100003 vertices, 8 per vertex: 1.02 -> 0.55 ms; 10007
+// vertices 0.143 -> 0.074 ms.
+template <class IT>
+__device__ __forceinline__ void mark_row_columns(const RowCtx<IT, NoVal>& cx, unsigned* bm, int w,
+                                                 int nwarps) {
+    const int lane = lane_id();
+    const IT* ciB = cx.ciB;
+    const bool shared = cx.a1 - cx.a0 <= 32LL * nwarps;
+    const int first = shared ? w : 0, step = shared ? nwarps : 1;
+    const long long stride = shared ? 32 : 32LL * nwarps;
+    for (long long b = cx.a0 + (shared ? 0 : 32LL * w); b < cx.a1; b += stride) {
+        long long lo = 0;
+        int len = 0;
+        if (b + lane < cx.a1) {
+            const long long k = (long long)cx.ciA[b + lane];
+            lo = cx.rpB[k];
+            len = (int)(cx.rpB[k + 1] - lo);
+        }
+        // rows of B of 32 entries and more, in pieces of 256
+        const int pieces = len >= 32 ? (len + 255) >> 8 : 0;
+        const int incl = warp_incl_scan(pieces);
+        const int before = incl - pieces;
+        const int total = __shfl_sync(kFull, incl, 31);
+        for (int p = first; p < total; p += step) {
+            // the last entry whose pieces start at or before p (one without
+            // pieces starts where the next does)
+            const int e = 31 - __clz(__ballot_sync(kFull, before <= p));
+            const int at = (p - __shfl_sync(kFull, before, e)) << 8;
+            const IT* cb = ciB + __shfl_sync(kFull, lo, e) + at + lane;
+            const int left = __shfl_sync(kFull, len, e) - at;
+            IT j[8];
+            if (left >= 256) {
+#pragma unroll
+                for (int t = 0; t < 8; ++t) j[t] = cb[32 * t];
+#pragma unroll
+                for (int t = 0; t < 8; ++t) atomicOr(&bm[j[t] >> 5], 1u << (j[t] & 31));
+            } else {
+#pragma unroll
+                for (int t = 0; t < 8; ++t) j[t] = 32 * t + lane < left ? cb[32 * t] : IT(-1);
+#pragma unroll
+                for (int t = 0; t < 8; ++t)
+                    if (j[t] >= 0) atomicOr(&bm[j[t] >> 5], 1u << (j[t] & 31));
+            }
+        }
+        // shorter ones, flattened: 128 products per step
+        const int slen = len < 32 ? len : 0;
+        if (__any_sync(kFull, slen > 0)) {
+            const int sincl = warp_incl_scan(slen);
+            const int sbefore = sincl - slen;
+            const int stotal = __shfl_sync(kFull, sincl, 31);
+            for (int f0 = 128 * first; f0 < stotal; f0 += 128 * step) {
+                IT j[4];
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                    const int f = f0 + 32 * t + lane;
+                    // the last entry that starts at or before f
+                    int e = 0;
+#pragma unroll
+                    for (int d = 16; d; d >>= 1)
+                        if (__shfl_sync(kFull, sbefore, e + d) <= f) e += d;
+                    const long long q =
+                        __shfl_sync(kFull, lo, e) + (f - __shfl_sync(kFull, sbefore, e));
+                    j[t] = f < stotal ? ciB[q] : IT(-1);
+                }
+#pragma unroll
+                for (int t = 0; t < 4; ++t)
+                    if (j[t] >= 0) atomicOr(&bm[j[t] >> 5], 1u << (j[t] & 31));
+            }
+        }
+    }
 }
 
 template <class IT, int MAXT, int MINB>
@@ -966,10 +1049,6 @@ __device__ __forceinline__ void symbolic_dense_kernel_body(const ProdDesc* __res
         if (rr >= nrows) break;
         const long long r = drow[rr];
         const RowCtx<IT, NoVal> cx = row_ctx<IT, NoVal>(D, rb, nprod, r);
-        const long long a0 = cx.a0, a1 = cx.a1;
-        const IT* ciA = cx.ciA;
-        const int64_t* rpB = cx.rpB;
-        const IT* ciB = cx.ciB;
         const int NW = (int)((cx.n + 31) >> 5);
         const int P = cx.P;
         if (NW > max_words) {  // n beyond the shared-memory bitmap: reported, row skipped
@@ -977,28 +1056,7 @@ __device__ __forceinline__ void symbolic_dense_kernel_body(const ProdDesc* __res
             group_sync(g, gthreads, groups);
             continue;
         }
-        for (long long b = a0 + (long long)w * 32; b < a1; b += (long long)nwarps * 32) {
-            const int nb = (int)min(32LL, a1 - b);
-            long long lo = 0;
-            int len = 0;
-            if (lane < nb) {
-                long long k = (long long)ciA[b + lane];
-                lo = rpB[k];
-                len = (int)(rpB[k + 1] - lo);
-            }
-            walk_batch4(nb, lo, len, [&](const long long (&q)[4], const int (&)[4],
-                                         const bool (&valid)[4], bool) {
-                long long j[4];
-#pragma unroll
-                for (int t = 0; t < 4; ++t) j[t] = valid[t] ? (long long)ciB[q[t]] : -1;
-                // one shared atomic per product: OR-ing the lanes' bits of a
-                // common word first (a segmented scan, or __match_any_sync with
-                // __reduce_or_sync) was measured 3x and 5x slower
-#pragma unroll
-                for (int t = 0; t < 4; ++t)
-                    if (j[t] >= 0) atomicOr(&bm[j[t] >> 5], 1u << (j[t] & 31));
-            });
-        }
+        mark_row_columns<IT>(cx, bm, w, nwarps);
         group_sync(g, gthreads, groups);
         long long part = 0;
         for (int c = w; c < P; c += nwarps) {

@@ -198,8 +198,8 @@ cudaError_t launch_symbolic(Plan& P, unsigned char* ws, int64_t* rowcnt) {
     if (dense) {
         // one block per row; the block size follows the bitmap: the most
         // resident warps, and among equals the smaller blocks (more rows in
-        // flight) -- 256 threads while six blocks fit, 1024 when only one does
-        auto ks = symbolic_dense_kernel<IT, 512, 3>;
+        // flight) -- 256 threads while several fit, 1024 when only one does
+        auto ks = symbolic_dense_kernel<IT, 512, 2>;
         auto kb = symbolic_dense_kernel<IT, 1024, 1>;
         const int max_words = (int)((std::min(P.max_n, P.max_dense_n) + 31) / 32);
         size_t smem = (size_t)max_words * 4;
