@@ -301,15 +301,17 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
     off += align_up((size_t)R * sizeof(int32_t));
     P->cap = (int64_t*)(P->pws + off);
 
+    // counters (zero), descriptors and row bases lie one after another and go up
+    // in one copy
     cudaStream_t s = P->stream;
-    cudaError_t e = cudaMemcpyAsync(P->d_descs, P->descs.data(), count * sizeof(sg::ProdDesc),
-                                    cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(P->rb, rb.data(), (count + 1) * sizeof(long long),
-                            cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(P->bb, bb.data(), (count + 1) * sizeof(long long),
-                            cudaMemcpyHostToDevice, s);
+    std::vector<unsigned char> head((size_t)((unsigned char*)(P->bb + count + 1) - P->pws), 0);
+    std::memcpy(head.data() + ((unsigned char*)P->d_descs - P->pws), P->descs.data(),
+                count * sizeof(sg::ProdDesc));
+    std::memcpy(head.data() + ((unsigned char*)P->rb - P->pws), rb.data(),
+                (count + 1) * sizeof(long long));
+    std::memcpy(head.data() + ((unsigned char*)P->bb - P->pws), bb.data(),
+                (count + 1) * sizeof(long long));
+    cudaError_t e = cudaMemcpyAsync(P->pws, head.data(), head.size(), cudaMemcpyHostToDevice, s);
     if (e != cudaSuccess) return bail(cuda_fail(e, "plan: descriptor upload"));
 
     auto prepare = [&]() -> cudaError_t {
@@ -331,8 +333,6 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
         return SPGEMM_OK;
     }
 
-    e = cudaMemsetAsync(P->cnt, 0, sizeof(sg::DevCounters), s);
-    if (e != cudaSuccess) return bail(cuda_fail(e, "plan: memset"));
     if (o.checked) {
         int* err = &P->cnt->err;
         for (int p = 0; p < count && e == cudaSuccess; ++p) {
@@ -545,15 +545,19 @@ spgemm_status spgemm_symbolic(spgemm_plan_t P, void* ws, size_t ws_bytes, int64_
                                               : sg::launch_symbolic<int64_t>(*P, w, rowptrC);
     if (e != cudaSuccess) return cuda_fail(e, "symbolic");
     sg::WsLayout L = sg::workspace_layout(*P);
-    e = sg::launch_exclusive_scan(rowptrC, P->R + 1, (int64_t*)(w + L.scan), s);
+    e = sg::launch_exclusive_scan(rowptrC, P->R + 1, (int64_t*)(w + L.scan), s, &P->cnt->nnz_c);
     if (e != cudaSuccess) return cuda_fail(e, "symbolic: scan");
-    int64_t total = 0;
-    int herr = 0;
-    SG_CUDA(cudaMemcpyAsync(&total, rowptrC + P->R, sizeof(int64_t), cudaMemcpyDeviceToHost, s),
-            "symbolic: readback");
-    SG_CUDA(cudaMemcpyAsync(&herr, &P->cnt->err, sizeof(int), cudaMemcpyDeviceToHost, s),
+    struct {
+        int64_t total;
+        int err;
+    } back{0, 0};
+    static_assert(offsetof(sg::DevCounters, err) == offsetof(sg::DevCounters, nnz_c) + 8,
+                  "total and error word are read back together");
+    SG_CUDA(cudaMemcpyAsync(&back, &P->cnt->nnz_c, 8 + sizeof(int), cudaMemcpyDeviceToHost, s),
             "symbolic: readback");
     SG_CUDA(cudaStreamSynchronize(s), "symbolic: sync");
+    const int64_t total = back.total;
+    const int herr = back.err;
     if (herr) return fail(SPGEMM_ERR_INTERNAL, "device check failed in symbolic phase (code %d)", herr);
     P->nnz_c = total;
     *nnz_c = total;

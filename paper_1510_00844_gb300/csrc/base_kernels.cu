@@ -1,5 +1,8 @@
 // Non-template kernels: row binning, int64 exclusive scan, empty rows; and
 // their host launchers.
+#include <map>
+#include <tuple>
+
 #include "plan.h"
 
 namespace sg {
@@ -90,10 +93,11 @@ __global__ void scan_partials_kernel(int64_t* part, long long nparts) {
     }
 }
 
-// part: the tiles' sums (direct), or the sums of the tiles before each.
+// part: the tiles' sums (direct), or the sums of the tiles before each.  The
+// last entry's result also goes to total_out, if given.
 __global__ void __launch_bounds__(kScanThreads)
     scan_apply_kernel(int64_t* __restrict__ x, long long N, const int64_t* __restrict__ part,
-                      bool direct) {
+                      bool direct, int64_t* total_out) {
     constexpr int kWarps = kScanThreads / 32;
     __shared__ long long ws[kWarps], before[kWarps];
     const int lane = lane_id(), w = threadIdx.x >> 5;
@@ -123,6 +127,7 @@ __global__ void __launch_bounds__(kScanThreads)
     for (int t = 0; t < kScanItems; ++t) {
         const long long incl = warp_incl_scan(v[t]);
         if (base + 32 * t < N) x[base + 32 * t] = carry + incl - v[t];
+        if (total_out && base + 32 * t == N - 1) *total_out = carry + incl - v[t];
         carry += __shfl_sync(kFull, incl, 31);
     }
 }
@@ -142,6 +147,22 @@ __global__ void product_rowptr_kernel(long long R, const long long* __restrict__
         const long long i = t - rb[lo] - lo;
         out[t] = g[rb[lo] + i] - g[rb[lo]];
     }
+}
+
+int occupancy_lookup(const void* kernel, int threads, size_t smem) {
+    thread_local std::map<std::tuple<int, const void*, int, size_t>, int> known;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    const auto key = std::make_tuple(dev, kernel, threads, smem);
+    const auto it = known.find(key);
+    if (it != known.end()) return it->second;
+    int b = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess ||
+        b < 1)
+        return 1;   // an error is not remembered
+    if (known.size() >= 256) known.clear();
+    known[key] = b;
+    return b;
 }
 
 cudaError_t launch_class_offsets(Plan& P) {
@@ -165,7 +186,8 @@ size_t scan_temp_bytes(long long N) {
     return (size_t)std::max<long long>(parts, 1) * sizeof(int64_t);
 }
 
-cudaError_t launch_exclusive_scan(int64_t* x, long long N, int64_t* temp, cudaStream_t s) {
+cudaError_t launch_exclusive_scan(int64_t* x, long long N, int64_t* temp, cudaStream_t s,
+                                  int64_t* total_out) {
     if (N <= 0) return cudaSuccess;
     long long parts = (N + kScanTile - 1) / kScanTile;
     const bool direct = parts <= kScanDirect;
@@ -178,7 +200,7 @@ cudaError_t launch_exclusive_scan(int64_t* x, long long N, int64_t* temp, cudaSt
         scan_partials_kernel<<<1, 1024, 0, s>>>(temp, parts);
     }
     count_launches(1);
-    scan_apply_kernel<<<(unsigned)parts, kScanThreads, 0, s>>>(x, N, temp, direct);
+    scan_apply_kernel<<<(unsigned)parts, kScanThreads, 0, s>>>(x, N, temp, direct, total_out);
     return cudaGetLastError();
 }
 

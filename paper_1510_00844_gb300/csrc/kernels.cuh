@@ -74,11 +74,12 @@ struct DevCounters {
     unsigned long long max_flops;
     unsigned long long work_counter[4];  // dynamic row grabbing
     unsigned long long max_dense_len;    // longest A row among dense rows
+    int64_t nnz_c;                       // total of the row pointers, read back with err
     int err;
     int unsupported;
     int seg_log2;                        // dense work-unit size of the plan
     unsigned blocks_done;                // of the row analysis
-    int pad[28];
+    int pad[26];
 };
 
 // Product owning global row r: the largest p with rb[p] <= r.

@@ -8,13 +8,13 @@
 
 namespace sg {
 
+// Resident blocks per SM.  A product asks for a dozen of these, always the same
+// while its sizes are; the answers (a function of the arguments and the device
+// alone) are remembered per thread, 256 at most.
+int occupancy_lookup(const void* kernel, int threads, size_t smem);
 template <class F>
 int occupancy_blocks(F kernel, int threads, size_t smem) {
-    int b = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess ||
-        b < 1)
-        b = 1;
-    return b;
+    return occupancy_lookup(reinterpret_cast<const void*>(kernel), threads, smem);
 }
 
 template <class F>
