@@ -103,7 +103,9 @@ typedef struct {
 typedef struct {
     int32_t semiring;        /* spgemm_semiring; OR_AND ignores values and yields a pattern */
     int32_t checked;         /* nonzero: validate A and B on the device before planning */
-    int32_t dense_chunk;     /* columns per dense-row chunk: 0 = library choice, 1024 or 2048 */
+    int32_t dense_chunk;     /* columns per dense-row chunk: 0 = library choice (1024 or 2048;
+                                128 to 1024 where a narrow product's longest row would
+                                otherwise make too few work units), 1024 or 2048 */
     int32_t dense_min_flops; /* rows with more products use dense accumulators:
                                 0 = 1024, else 32..1024 (autotuned knob) */
     int32_t max_row_nnz;     /* device-sized plans: bound on the entries of a dense row of A
@@ -133,9 +135,10 @@ typedef struct {
     int64_t flops;          /* total multiplications */
     int64_t max_row_flops;
     int64_t rows_empty;     /* rows with no products */
-    int64_t rows_hash;      /* rows handled with per-warp hash tables */
+    int64_t rows_hash;      /* rows of at most dense_min_flops products (sorted in registers,
+                               ranked by a bitmap or hashed, by size) */
     int64_t rows_dense;     /* rows handled with column-chunked dense accumulators */
-    int64_t chunk_width;    /* columns per dense chunk */
+    int64_t chunk_width;    /* columns per dense chunk (may be narrower than 1024) */
     int64_t chunks_per_row; /* dense chunks per dense row */
     int64_t nnz_c;          /* set by spgemm_symbolic, -1 before */
 } spgemm_info;
@@ -354,7 +357,9 @@ spgemm_status spgemm_learned_multiply(const spgemm_csr* A, const spgemm_csr* B,
 spgemm_status spgemm_plan_info(spgemm_plan_t plan, spgemm_info* info);
 
 /* Device workspace (bytes) that spgemm_symbolic / spgemm_numeric need for
- * this plan (dense-chunk counts and per-entry cursors).  Host call. */
+ * this plan (dense-chunk counts and per-entry cursors; for OR_AND also a
+ * bitmap of n bits per dense row while all of them take at most a byte per
+ * product and 8 GB).  Host call. */
 spgemm_status spgemm_workspace_size(spgemm_plan_t plan, size_t* bytes);
 
 /* spgemm_symbolic -- count the nonzeros of every row of C (the size of the

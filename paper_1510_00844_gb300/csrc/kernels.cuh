@@ -5,14 +5,20 @@
 //
 // Row classes (decided from flops_i = sum_{k in A(i,:)} nnz(B(k,:)), Sec. 2):
 //   EMPTY       flops_i == 0
-//   HASH(b)     flops_i <= dense_min (<= 1024): one warp per row, warp-private
-//               hash table in shared memory (keys for the symbolic phase, keys
-//               + values for the numeric phase), output sorted in the warp
-//               (bitonic sort up to 64 entries, stable radix sort above).
+//   HASH(b)     flops_i <= dense_min (<= 1024).  Up to 32 products: one warp
+//               per row in registers (equal columns by match).  33 to 128 and n
+//               < 2^25, numeric: one warp per row, products sorted in
+//               registers by (column, position).  129 to 1024 and n within
+//               rank_max_n, outside the persistent chain: one block per row,
+//               columns ranked by a bitmap of n bits in shared memory.
+//               Otherwise: one warp per row with a warp-private hash table in
+//               shared memory, output sorted in the warp (bitonic sort up to
+//               64 entries, stable radix sort above).
 //   DENSE(b)    flops_i > dense_min: symbolic = one block per row with a
 //               bitmap of all n columns in shared memory (also yields
-//               per-chunk counts); numeric = one warp per (row, column
-//               segment) sweeping column chunks of width W with a dense
+//               per-chunk counts; kept in the workspace for patterns, whose
+//               numeric phase writes the columns from it); numeric = one warp
+//               per (row, column segment) sweeping column chunks with a dense
 //               accumulator, so the output comes out sorted.  DENSE rows are
 //               bucketed by floor(log2 flops_i), largest first.
 #pragma once
