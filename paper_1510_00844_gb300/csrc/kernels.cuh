@@ -8,9 +8,11 @@
 //   HASH(b)     flops_i <= dense_min (<= 1024).  Up to 32 products: one warp
 //               per row in registers (equal columns by match).  33 to 128 and n
 //               < 2^25, numeric: one warp per row, products sorted in
-//               registers by (column, position).  129 to 1024 and n within
-//               rank_max_n, outside the persistent chain: one block per row,
-//               columns ranked by a bitmap of n bits in shared memory.
+//               registers by (column, position); likewise 129 to 512 and n <
+//               2^23 outside the persistent chain and predicted slots.  Other
+//               rows of 129 to 1024 and n within rank_max_n, outside the
+//               chain: one block per row, columns ranked by a bitmap of n bits
+//               in shared memory.
 //               Otherwise: one warp per row with a warp-private hash table in
 //               shared memory, output sorted in the warp (bitonic sort up to
 //               64 entries, stable radix sort above).
@@ -1600,7 +1602,8 @@ struct __align__(16) DenseRun {
 };
 
 // ------------------------- rows of 129 to 1024 products, ranked by a bitmap
-// Hash bins 2 and 3 in products of at most rank_max_n columns.  A block of four
+// Hash bins 2 (counts, and slots of predicted size) and 3 in products of at most
+// rank_max_n columns.  A block of four
 // warps takes a row; product f of the row (ascending k) sits in warp (f / 32) %
 // 4, lane f % 32, item f / 128.  The products set the bits of their columns;
 // the set bits before a column are its place in C(i,:), so nothing is hashed or
@@ -1911,6 +1914,225 @@ __global__ void __launch_bounds__(32 * kRankWarps)
         }
         rank_clear(bits, nwords);
         __syncthreads();
+    }
+}
+
+// ------------------------------ rows of 129 to 512 products, sorted by a warp
+// Hash bin 2 outside slot mode.  As for the shorter rows, the products' (column,
+// place) keys are sorted in registers and each run of equal columns is added up
+// by the lane of its first key, in ascending place; eight or sixteen keys per
+// lane.  Nine bits hold the place, so columns must be below 2^23.
+// What bounds it: instructions (about two of sorting per product) and the
+// gathers of the values, at 32 warps per SM where the table in float64 held 16.
+// Against the table and the bitmap, Erdos-Renyi squares of 16 per column,
+// numeric in us, float64 and float32: 8192 columns bitmap 42 and 39, sorted 34
+// and 36; 32768 columns bitmap 160 and 143, sorted 114 and 108; 65536 columns
+// table 358 and 288, sorted 220 and 213; 262144 columns table 1581 and 1248,
+// sorted 925 and 844.  64 uneven products in float32: 2550 -> 2130.
+constexpr int kSort9Bits = 9;
+constexpr int kSort9Most = 1 << kSort9Bits;
+constexpr int kSort9Warps = 8;
+constexpr long long kSort9MaxN = 1LL << (32 - kSort9Bits);
+
+// Per warp: values by place, sorted keys (a word of padding per lane), runs.
+template <class V>
+constexpr size_t sort9_warp_bytes() {
+    return (VOps<V>::has_val ? kSort9Most * sizeof(V) : 0) + (kSort9Most + 32) * sizeof(unsigned) +
+           32 * sizeof(DenseRun<V>);
+}
+
+// Ascending sort of 32 * ITEMS keys, key lane * ITEMS + t in item t: a bitonic
+// network whose merges begin with a mirrored exchange, so every exchange puts
+// the smaller key first and those within a lane are a min and a max.  Fifteen
+// levels of exchanges between lanes, whatever ITEMS is.
+template <int ITEMS>
+__device__ __forceinline__ void warp_sort_blocked(unsigned (&key)[ITEMS]) {
+    const int lane = lane_id();
+    auto within = [&](int t, int o) {
+        const unsigned x = min(key[t], key[o]), y = max(key[t], key[o]);
+        key[t] = x;
+        key[o] = y;
+    };
+#pragma unroll
+    for (int k = 2; k <= 32 * ITEMS; k <<= 1) {
+        if (k <= ITEMS) {
+#pragma unroll
+            for (int t = 0; t < ITEMS; ++t)
+                if ((t ^ (k - 1)) > t) within(t, t ^ (k - 1));
+        } else {
+            const int m = k / ITEMS - 1;
+            const bool lower = (lane & (k / ITEMS / 2)) == 0;
+#pragma unroll
+            for (int t = 0; t < ITEMS / 2; ++t) {
+                const int o = ITEMS - 1 - t;
+                const unsigned x = __shfl_xor_sync(kFull, key[o], m);
+                const unsigned y = __shfl_xor_sync(kFull, key[t], m);
+                key[t] = lower ? min(key[t], x) : max(key[t], x);
+                key[o] = lower ? min(key[o], y) : max(key[o], y);
+            }
+        }
+#pragma unroll
+        for (int j = k >> 2; j > 0; j >>= 1) {
+            if (j >= ITEMS) {
+                const bool lower = (lane & (j / ITEMS)) == 0;
+#pragma unroll
+                for (int t = 0; t < ITEMS; ++t) {
+                    const unsigned y = __shfl_xor_sync(kFull, key[t], j / ITEMS);
+                    key[t] = lower ? min(key[t], y) : max(key[t], y);
+                }
+            } else {
+#pragma unroll
+                for (int t = 0; t < ITEMS; ++t)
+                    if ((t ^ j) > t) within(t, t ^ j);
+            }
+        }
+    }
+}
+
+// Sorts the first 32 * ITEMS keys and leaves key i in sorted[i + i / ITEMS]
+// (no bank conflicts on the way in).
+template <int ITEMS, int N>
+__device__ __forceinline__ void sort9_store(const unsigned (&key)[N], unsigned* sorted) {
+    unsigned k[ITEMS];
+#pragma unroll
+    for (int t = 0; t < ITEMS; ++t) k[t] = key[t];
+    warp_sort_blocked<ITEMS>(k);
+#pragma unroll
+    for (int t = 0; t < ITEMS; ++t) sorted[lane_id() * (ITEMS + 1) + t] = k[t];
+}
+
+template <class IT, class V>
+__global__ void __launch_bounds__(32 * kSort9Warps)
+    numeric_sort_kernel(const ProdDesc* __restrict__ D, const long long* __restrict__ rb,
+                        int nprod, const int32_t* __restrict__ rows, const DevCounters* cnt,
+                        int cls, const int64_t* __restrict__ rpC, long long cap,
+                        IT* __restrict__ ciC, V* __restrict__ vC, int* err) {
+    constexpr bool HV = VOps<V>::has_val;
+    constexpr bool kPlain = std::is_same<V, double>::value || std::is_same<V, float>::value ||
+                            std::is_same<V, int64_t>::value;
+    constexpr int B = kSort9Bits;
+    constexpr int N = kSort9Most / 32;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int lane = lane_id(), w = threadIdx.x >> 5;
+    unsigned char* base = smem_raw + w * sort9_warp_bytes<V>();
+    DenseRun<V>* runs = reinterpret_cast<DenseRun<V>*>(base);
+    V* vals = reinterpret_cast<V*>(base + 32 * sizeof(DenseRun<V>));
+    unsigned* sorted = reinterpret_cast<unsigned*>(base + 32 * sizeof(DenseRun<V>) +
+                                                   (HV ? kSort9Most * sizeof(V) : 0));
+    const long long nrows = (long long)cnt->class_count[cls];
+    const int32_t* crow = rows + cnt->class_off[cls];
+    for (long long rr = (long long)blockIdx.x * kSort9Warps + w; rr < nrows;
+         rr += (long long)gridDim.x * kSort9Warps) {
+        const long long r = crow[rr];
+        const RowCtx<IT, V> c = row_ctx<IT, V>(D, rb, nprod, r);
+        const long long out = rpC[r];
+        const long long room = rpC[r + 1] - out;
+        unsigned key[N];
+#pragma unroll
+        for (int t = 0; t < N; ++t) key[t] = 0xffffffffu;
+        int np = 0;
+        for (long long b = c.a0; b < c.a1; b += 32) {
+            const int nb = (int)min(32LL, c.a1 - b);
+            long long lo = 0;
+            int len = 0;
+            DenseRun<V> run{};
+            if (lane < nb) {
+                const long long k = (long long)c.ciA[b + lane];
+                lo = c.rpB[k];
+                len = (int)min(c.rpB[k + 1] - lo, (long long)kSort9Most);
+                if constexpr (HV) run.a = load_val(c.vA, b + lane);
+            }
+            const int incl = warp_incl_scan(len);
+            const int tot = min(__shfl_sync(kFull, incl, 31), kSort9Most - np);
+            if (tot <= 0) continue;
+            const int start = np + incl - len;
+            const unsigned some = __ballot_sync(kFull, len > 0);
+            run.off = lo - start;
+            __syncwarp();   // the table's last use is over
+            if (len > 0) runs[__popc(some & lanemask_lt())] = run;
+            __syncwarp();
+#pragma unroll
+            for (int t = 0; t < N; ++t) {
+                if (32 * t >= np + tot || 32 * t + 32 <= np) continue;
+                // the run of product f: the runs that start at or before it
+                const unsigned M = __reduce_or_sync(
+                    kFull,
+                    len > 0 && start >= 32 * t && start < 32 * t + 32 ? 1u << (start - 32 * t) : 0u);
+                const int e = __popc(__ballot_sync(kFull, len > 0 && start < 32 * t)) +
+                              __popc(M & lanemask_le()) - 1;
+                const int f = 32 * t + lane;
+                if (f >= np && f < np + tot) {
+                    const DenseRun<V> x = runs[e];
+                    const long long q = x.off + f;
+                    key[t] = (unsigned)c.ciB[q] << B | (unsigned)f;
+                    if constexpr (HV) vals[f] = VOps<V>::mul(x.a, load_val(c.vB, q));
+                }
+            }
+            np += tot;
+        }
+        const int sh = np <= 256 ? 3 : 4;   // log2 of the keys per lane
+        if (np <= 256) sort9_store<8>(key, sorted);
+        else sort9_store<16>(key, sorted);
+        __syncwarp();
+        int count = 0;
+        for (int t0 = 0; t0 < np; t0 += 128) {
+            unsigned x[4];
+            V sum[4];
+            int pos[4];
+            bool more[4];
+            unsigned heads = 0u;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = t0 + 32 * u + lane;
+                bool head = false;
+                x[u] = 0u;
+                if (i < np) {
+                    x[u] = sorted[i + (i >> sh)];
+                    head = i == 0 || sorted[i - 1 + ((i - 1) >> sh)] >> B != x[u] >> B;
+                }
+                const unsigned m = __ballot_sync(kFull, head);
+                pos[u] = count + __popc(m & lanemask_lt());
+                count += __popc(m);
+                heads |= head ? 1u << u : 0u;
+                more[u] = head;
+                sum[u] = VOps<V>::init();
+                if constexpr (HV) {
+                    if (head) {
+                        const V v = vals[x[u] & (kSort9Most - 1)];
+                        // the identity plus v is v, bit for bit, for (+, x)
+                        if constexpr (kPlain) sum[u] = v;
+                        else sum[u] = VOps<V>::add(sum[u], v);
+                    }
+                }
+            }
+            if constexpr (HV) {
+                for (int d = 1;; ++d) {
+                    bool any = false;
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int i = t0 + 32 * u + lane + d;
+                        unsigned y = 0u;
+                        more[u] = more[u] && i < np;
+                        if (more[u]) y = sorted[i + (i >> sh)];
+                        more[u] = more[u] && y >> B == x[u] >> B;
+                        if (more[u]) sum[u] = VOps<V>::add(sum[u], vals[y & (kSort9Most - 1)]);
+                        any = any || more[u];
+                    }
+                    if (!__any_sync(kFull, any)) break;
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if ((heads >> u & 1u) && pos[u] < room && out + pos[u] < cap) {
+                    ciC[out + pos[u]] = (IT)(x[u] >> B);
+                    if constexpr (HV) vC[out + pos[u]] = sum[u];
+                }
+        }
+        if (lane == 0) {
+            if (count != room) atomicExch(err, (int)kDevCountMismatch);
+            if (out + room > cap) atomicExch(err, (int)kDevCapacity);
+        }
+        __syncwarp();   // the keys and values have been read: the next row may write them
     }
 }
 

@@ -137,6 +137,29 @@ cudaError_t num_rank_bin(Plan& P, int bin, long long nrows, const int64_t* rpC, 
     return cudaGetLastError();
 }
 
+// Bin 2's numeric pass sorts in registers, which was faster than bitmap and
+// table at every width (4096 to 262144 columns, figures at the kernel), unless
+// its slots were predicted: a row may then have more products than the bin's
+// bound.
+inline bool sort_bin(const Plan& P, int bin) {
+    return bin == 2 && !P.prm && P.max_n < kSort9MaxN;
+}
+
+template <class IT, class V>
+cudaError_t num_sort_bin(Plan& P, int bin, long long nrows, const int64_t* rpC, long long cap,
+                         IT* colC, V* valC) {
+    auto k = numeric_sort_kernel<IT, V>;
+    const size_t smem = kSort9Warps * sort9_warp_bytes<V>();
+    cudaError_t e = allow_smem(k, smem);
+    if (e != cudaSuccess) return e;
+    const int occ = occupancy_blocks(k, 32 * kSort9Warps, smem);
+    count_launches(1);
+    k<<<(unsigned)class_grid(P, nrows, kSort9Warps, occ), 32 * kSort9Warps, smem, P.stream>>>(
+        P.d_descs, P.rb, P.nprod, P.rows, P.cnt, kClassHash0 + bin, rpC, cap, colC, valC,
+        &P.cnt->err);
+    return cudaGetLastError();
+}
+
 template <class IT, int LOG2T, int WARPS>
 cudaError_t sym_hash_bin(Plan& P, int bin, int64_t* rowcnt) {
     using K = typename KeyT<IT>::type;
@@ -240,6 +263,8 @@ cudaError_t num_hash_bin(Plan& P, int bin, const int64_t* rpC, long long cap, IT
     if (!P.device_sized && nrows == 0) return cudaSuccess;
     if (P.device_sized && bin > 0 && (hash_bin_flops(bin - 1) >> P.hash_shift) >= P.dense_min)
         return cudaSuccess;
+    if (!rowend && sort_bin(P, bin))
+        return num_sort_bin<IT, V>(P, bin, nrows, rpC, cap, colC, valC);
     if (rank_bin(P, bin, false))
         return num_rank_bin<IT, V>(P, bin, nrows, rpC, cap, colC, valC, rowend, overflow,
                                    overflow_count);

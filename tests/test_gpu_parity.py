@@ -588,3 +588,41 @@ def test_pattern_of_dense_rows(sg, n, rows, l, density, index):
         sg.check(p)
         assert np.array_equal(rp.cpu().numpy(), R.rowptr)
         assert np.array_equal(col.cpu().numpy().astype(np.int64), R.col)
+
+
+@pytest.mark.parametrize("value", ["u01_f64", "u11_f32", "int", "none"])
+@pytest.mark.parametrize("n", [700, 2**23 - 1, 2**23])
+def test_rows_of_129_to_512_products_sorted(sg, n, value):
+    """Rows on both sides of eight and sixteen keys per lane, with distinct
+    columns, with columns that most B rows share and with the last column, on
+    both sides of the width up to which a warp sorts them."""
+    rng = np.random.default_rng(n % 1000 + len(value))
+    lens = [0] * 8 + [1] * 300 + [3, 17, 32, 33, 63, 64, 100, 128] * 3
+    cols = []
+    for t, k in enumerate(lens):
+        c = [rng.choice(n, k, replace=False), np.arange(k), n - k + np.arange(k)][t % 3]
+        cols.append(np.sort(c))
+    size = np.array([c.size for c in cols])
+    B = inputs.CSR(len(cols), n, np.concatenate([[0], np.cumsum(size)]).astype(np.int64),
+                   np.concatenate(cols).astype(np.int32),
+                   inputs.draw_values(rng, int(size.sum()), value))
+    rows = []
+    for target in [129, 160, 161, 255, 256, 257, 288, 289, 511, 512]:
+        for most in (1, 40, 128):
+            pick, left = [], target
+            for k in rng.permutation(len(cols)):
+                if size[k] <= min(left, most):
+                    pick.append(k)
+                    left -= size[k]
+            rows.append(np.sort(pick))
+    colA = np.concatenate(rows).astype(np.int32)
+    rpA = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
+    A = inputs.CSR(len(rows), len(cols), rpA, colA, inputs.draw_values(rng, colA.size, value))
+    sr = 1 if value == "none" else 0
+    C = run(sg, A, B, semiring=sr)
+    R = oracle.spgemm(A, B, semiring="or_and" if sr else "plus_times")
+    assert_pattern_equal(C, R)
+    if value == "u11_f32":
+        assert_values_close(C, R, A, B, "f32")
+    elif value != "none":
+        assert np.array_equal(C.to_host()[2], R.val)
