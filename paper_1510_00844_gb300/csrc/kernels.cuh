@@ -1106,12 +1106,14 @@ __global__ void __launch_bounds__(MAXT, MINB) symbolic_dense_kernel(const ProdDe
 
 // The columns of the dense rows of a pattern from the bitmaps the symbolic
 // pass kept (max_words words per dense row): a block per row, each warp a range of
-// chunks; the chunks' counts give its place in C(i,:).  A lane takes a word and
-// puts its bits' offsets into the warp's stage, so that the stores to C are
-// coalesced.  What bounds it: DRAM (the bitmaps once, C once), where sweeping
-// the products of every row again took as long as their symbolic pass: R-MAT,
-// 100003 vertices (233 M columns) 1.82 -> 0.63 ms.
-constexpr int kColStage = 512;   // of the 1024 columns of 32 words
+// chunks; the chunks' counts give its place in C(i,:).  A lane takes four words
+// and puts their bits' offsets into the warp's stage, highest first (one
+// instruction of the slow pipe per bit), so that the stores to C are coalesced.
+// What bounds it: DRAM traffic (the bitmaps once, C once) in part and the bit
+// loops; sweeping the products of every row again took as long as their symbolic
+// pass.  R-MAT, 100003 vertices (233 M columns): sweep 1.82 ms, a word per lane
+// and a scan for each 0.63 ms, four 0.59 ms; loading a step ahead 0.60 ms.
+constexpr int kColStage = 512;   // of the 4096 columns of 128 words
 template <class IT>
 __global__ void __launch_bounds__(256)
     dense_columns_kernel(const ProdDesc* __restrict__ D, const long long* __restrict__ rb,
@@ -1147,33 +1149,32 @@ __global__ void __launch_bounds__(256)
         const int t1 = min(NW, ce * chunk_words);
         for (int b = cs * chunk_words; b < t1; b += 128) {
             unsigned word[4];
+            int pc = 0;
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const int t = b + 32 * u + lane;
+                const int t = b + 4 * lane + u;
                 word[u] = t < t1 ? words[t] : 0u;
+                pc += __popc(word[u]);
             }
+            const int incl = warp_incl_scan(pc);
+            const int total = __shfl_sync(kFull, incl, 31);
+            int p = incl - 1;   // the place of this lane's highest bit left
+            for (int to = total; to > 0; to -= kColStage) {
+                const int from = max(0, to - kColStage);
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int pc = __popc(word[u]);
-                const int incl = warp_incl_scan(pc);
-                const int total = __shfl_sync(kFull, incl, 31);
-                // two halves of the lanes when the words hold more than the stage
-                const int first = total <= kColStage ? total : __shfl_sync(kFull, incl, 15);
-                for (int h = 0; h < 2; ++h) {
-                    const int from = h == 0 ? 0 : first, to = h == 0 ? first : total;
-                    if (from == to) continue;
-                    if (total <= kColStage || (lane >> 4) == h) {
-                        int p = incl - pc - from;
-                        for (; word[u]; word[u] &= word[u] - 1u)
-                            stage[p++] = (unsigned short)(lane * 32 + __ffs(word[u]) - 1);
+                for (int u = 3; u >= 0; --u)
+                    while (word[u] && p >= from) {
+                        const int bit = 31 - __clz(word[u]);
+                        stage[p - from] = (unsigned short)(lane * 128 + u * 32 + bit);
+                        word[u] ^= 1u << bit;
+                        --p;
                     }
-                    __syncwarp();
-                    for (int x = lane; x < to - from; x += 32)
-                        dst[from + x] = (IT)((long long)(b + 32 * u) * 32 + stage[x]);
-                    __syncwarp();
-                }
-                dst += total;
+                __syncwarp();
+                for (int x = from + lane; x < to; x += 32)
+                    dst[x] = (IT)((long long)b * 32 + stage[x - from]);
+                __syncwarp();
             }
+            dst += total;
         }
     }
 }
