@@ -296,9 +296,9 @@ def _timed(torch, fn, reps):
 
 def merge_roofline(sg, torch, dA, c=4, reps=3):
     """The multiway merge alone on the 4 k-slice partials of the product
-    (count + scan + numeric, then the numeric pass by itself), register
-    windows against lists staged in shared memory by bulk asynchronous
-    copies.  Algorithmic bytes of the numeric pass: every partial entry read
+    (count + scan + numeric, then the numeric pass by itself), the default
+    form (reported as "windows") against lists staged in shared memory by
+    bulk asynchronous copies.  Algorithmic bytes of the numeric pass: every partial entry read
     once and every entry of C written once (index + value each), plus the c
     partial row-pointer arrays and rowptr(C)."""
     _, parts = sg.spgemm_kslice(dA, dA, c)
