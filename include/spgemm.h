@@ -488,7 +488,9 @@ size_t spgemm_merge_workspace_size(int32_t c, int64_t m, int64_t n);
  * (sorted rows).  Writes rowptrC (int64[m+1]) of C = sum_s parts[s] and
  * nnz(C) (host).  Waits for the stream.  Each part's nnz must be the length of its
  * col array (as stated for spgemm_csr): a row of more than 8192 entries over
- * all parts is cut into segments only if they can hold that many. */
+ * all parts is cut into segments only if they can hold that many.  A row that
+ * does not ascend may be found (INVALID_CSR) or give a wrong sum; the call ends
+ * and writes inside its arrays either way. */
 spgemm_status spgemm_merge_symbolic(int32_t c, const spgemm_csr* parts, const spgemm_opts* opts,
                                     void* stream, void* ws, size_t ws_bytes, int64_t* rowptrC,
                                     int64_t* nnz_c);
@@ -520,8 +522,8 @@ spgemm_status spgemm_merge_symbolic_static(int32_t c, const spgemm_csr* parts,
                                            int64_t* rowptrC, int64_t* nnz_c);
 
 /* Reads the device error word the merge calls record in `ws` (waits for the
- * stream); SPGEMM_ERR_INTERNAL if a row's emitted count disagreed with
- * rowptrC. */
+ * stream); SPGEMM_ERR_INVALID_CSR if a part's row was found not to ascend,
+ * SPGEMM_ERR_INTERNAL if a row's emitted count disagreed with rowptrC. */
 spgemm_status spgemm_merge_check(void* stream, void* ws);
 
 #ifdef __cplusplus

@@ -468,7 +468,26 @@ spgemm_status check_merge_parts(int32_t c, const spgemm_csr* parts, const spgemm
     *vt_out = vt;
     return SPGEMM_OK;
 }
+
+// The status of a merge's nonzero device error word.
+spgemm_status merge_failed(int herr) {
+    if (herr == kDevBadIndex)
+        return fail(SPGEMM_ERR_INVALID_CSR, "a row of a part has unsorted or duplicate columns");
+    if (herr == kDevWaitTimeout)
+        return fail(SPGEMM_ERR_TIMEOUT, "a staged merge waited longer than its bound for a copy");
+    return fail(SPGEMM_ERR_INTERNAL, "device check failed in merge (code %d)", herr);
+}
 }  // namespace sg
+
+// The total of the row pointers and the error word, read back in one copy.
+struct CountReadback {
+    int64_t total = 0;
+    int err = 0;
+};
+constexpr size_t kCountReadbackBytes = 8 + sizeof(int);
+static_assert(offsetof(sg::DevCounters, err) == offsetof(sg::DevCounters, nnz_c) + 8 &&
+                  offsetof(CountReadback, err) == 8,
+              "total and error word lie side by side");
 
 extern "C" {
 
@@ -547,13 +566,8 @@ spgemm_status spgemm_symbolic(spgemm_plan_t P, void* ws, size_t ws_bytes, int64_
     sg::WsLayout L = sg::workspace_layout(*P);
     e = sg::launch_exclusive_scan(rowptrC, P->R + 1, (int64_t*)(w + L.scan), s, &P->cnt->nnz_c);
     if (e != cudaSuccess) return cuda_fail(e, "symbolic: scan");
-    struct {
-        int64_t total;
-        int err;
-    } back{0, 0};
-    static_assert(offsetof(sg::DevCounters, err) == offsetof(sg::DevCounters, nnz_c) + 8,
-                  "total and error word are read back together");
-    SG_CUDA(cudaMemcpyAsync(&back, &P->cnt->nnz_c, 8 + sizeof(int), cudaMemcpyDeviceToHost, s),
+    CountReadback back;
+    SG_CUDA(cudaMemcpyAsync(&back, &P->cnt->nnz_c, kCountReadbackBytes, cudaMemcpyDeviceToHost, s),
             "symbolic: readback");
     SG_CUDA(cudaStreamSynchronize(s), "symbolic: sync");
     const int64_t total = back.total;
@@ -683,13 +697,14 @@ spgemm_status spgemm_merge_symbolic(int32_t c, const spgemm_csr* parts, const sp
                                      (sg::MergeLong*)((unsigned char*)temp +
                                                       align_up(sg::scan_temp_bytes(m + 1))));
     if (e != cudaSuccess) return cuda_fail(e, "merge symbolic");
-    e = sg::launch_exclusive_scan(rowptrC, m + 1, temp, s);
+    e = sg::launch_exclusive_scan(rowptrC, m + 1, temp, s, &cnt->nnz_c);
     if (e != cudaSuccess) return cuda_fail(e, "merge symbolic: scan");
-    int64_t total = 0;
-    SG_CUDA(cudaMemcpyAsync(&total, rowptrC + m, sizeof(int64_t), cudaMemcpyDeviceToHost, s),
+    CountReadback back;
+    SG_CUDA(cudaMemcpyAsync(&back, &cnt->nnz_c, kCountReadbackBytes, cudaMemcpyDeviceToHost, s),
             "merge: readback");
     SG_CUDA(cudaStreamSynchronize(s), "merge: sync");
-    *nnz_c = total;
+    if (back.err) return sg::merge_failed(back.err);
+    *nnz_c = back.total;
     return SPGEMM_OK;
 }
 
@@ -729,10 +744,7 @@ spgemm_status spgemm_merge_check(void* stream, void* ws) {
     SG_CUDA(cudaMemcpyAsync(&herr, &((sg::DevCounters*)ws)->err, sizeof(int), cudaMemcpyDeviceToHost,
                             (cudaStream_t)stream), "merge check");
     SG_CUDA(cudaStreamSynchronize((cudaStream_t)stream), "merge check");
-    if (herr == sg::kDevWaitTimeout)
-        return fail(SPGEMM_ERR_TIMEOUT, "a staged merge waited longer than its bound for a copy");
-    if (herr) return fail(SPGEMM_ERR_INTERNAL, "device check failed in merge (code %d)", herr);
-    return SPGEMM_OK;
+    return herr ? sg::merge_failed(herr) : SPGEMM_OK;
 }
 
 }  // extern "C"

@@ -20,9 +20,9 @@
 // values) at 20 warps per SM, then DRAM.  The sweep of 1024-column chunks that
 // this replaces met few entries per chunk on rows of ordinary length and left
 // the longest rows to single warps.  Before and now: four lists of 100003-vertex
-// R-MAT graphs (3.3 GB read and written) 5.70 and 2.90 ms; the four partial
-// products of a 65536-vertex graph squared (11 GB) 8.9 and 7.3 ms; nine
-// partial products 40.6 and 13.4 ms.
+// R-MAT graphs (3.3 GB read and written) 5.70 and 2.80 ms; the four partial
+// products of a 65536-vertex graph squared (11 GB) 8.9 and 7.1 ms; nine
+// partial products 40.6 and 13.0 ms.
 #include <type_traits>
 
 #include "plan.h"
@@ -69,7 +69,12 @@ struct MergeWarp {
 
 // One row's (or segment's) merge by a warp: lane s holds list s's range
 // [cur, end).  Returns the number of outputs; writes them from `out` on
-// (numeric; never at or past out_end).
+// (numeric; never at or past out_end).  Rows must ascend; a row that does not
+// gives a wrong sum, or -1 where a chunk could take nothing.  Whatever the columns
+// are, every chunk takes an entry, only offsets below the span reach the map and
+// the list, and a value's place is below the chunk's outputs.  (Testing every 32
+// entries for the order cost 11 % of a merge of four 100003-vertex graphs,
+// testing for columns below c0 17 %; these bounds cost nothing.)
 template <class IT, class V, bool NUMERIC>
 __device__ __forceinline__ long long merge_range(int c, const MergeParts<IT, V>& parts,
                                                  long long cur, long long end, long long out,
@@ -84,13 +89,14 @@ __device__ __forceinline__ long long merge_range(int c, const MergeParts<IT, V>&
     unsigned short* list = reinterpret_cast<unsigned short*>(smem + L::kListAt);
     unsigned short* outs = reinterpret_cast<unsigned short*>(smem + L::kOutAt);
     const int lane = lane_id();
+    using U = typename std::make_unsigned<IT>::type;
     const IT* mycol = lane < c ? parts.col[lane] : nullptr;
     long long count = 0;
     // each list's share of the next chunk, its first column and the column
     // after its share: loaded as soon as the chunk before has taken its part
     long long total = 0, share = 0, head = kFar, next = kFar;
     auto offer = [&]() {
-        const long long left = end - cur;
+        const long long left = max(0LL, end - cur);
         total = warp_sum(left);
         share = left;
         if (total > L::kS) share = min(left, (long long)(L::kS - 8 * c) * left / total + 8);
@@ -101,6 +107,8 @@ __device__ __forceinline__ long long merge_range(int c, const MergeParts<IT, V>&
     while (total > 0) {
         const long long c0 = warp_min(head);
         const long long c1 = min(warp_min(next), c0 + kMergeSpan);
+        if (c1 <= c0) return -1;
+        const U width = (U)(c1 - c0);
         // columns: bits of the map, offsets in list order; four lists' loads
         // are in flight together
         int mine = 0;     // entries of list `lane` in the chunk
@@ -131,10 +139,11 @@ __device__ __forceinline__ long long merge_range(int c, const MergeParts<IT, V>&
                     int got = 0;
 #pragma unroll
                     for (int t = 0; t < 4; ++t) {
-                        const bool in =
-                            x0 + 32 * t + lane < lim[u] && (long long)j[u][t] < c1;
+                        // a column below c0 wraps around to far above the width
+                        const U off = (U)j[u][t] - (U)c0;
+                        const bool in = x0 + 32 * t + lane < lim[u] && off < width;
                         if (in) {
-                            const int d = (int)((long long)j[u][t] - c0);
+                            const int d = (int)off;
                             atomicOr(&bits[d >> 5], 1u << (d & 31));
                             if constexpr (HV) list[base + x0 + 32 * t + lane] = (unsigned short)d;
                             top = max(top, d + 1);
@@ -206,8 +215,10 @@ __device__ __forceinline__ long long merge_range(int c, const MergeParts<IT, V>&
                             const int x = x0 + 32 * t + lane;
                             if (x < n[u]) {
                                 const int d = list[base + x];
-                                const int slot = before[d >> 5] +
-                                                 __popc(bits[d >> 5] & ~(0xffffffffu << (d & 31)));
+                                const int slot =
+                                    min((int)before[d >> 5] +
+                                            __popc(bits[d >> 5] & ~(0xffffffffu << (d & 31))),
+                                        n_out - 1);
                                 if (kStoreFirst<V> && s0 + u == 0) acc[slot] = v[u][t];
                                 else acc[slot] = VOps<V>::add(acc[slot], v[u][t]);
                                 outs[slot] = (unsigned short)d;
@@ -253,6 +264,13 @@ __device__ __forceinline__ unsigned char* merge_warp_memory(unsigned char* smem_
     }
     unsigned* bits = reinterpret_cast<unsigned*>(smem + L::kBitsAt);
     for (int t = lane_id(); t < L::kWords; t += 32) bits[t] = 0u;
+    if constexpr (NUMERIC) {
+        // offsets and places that no chunk has written are in bounds too
+        unsigned short* before = reinterpret_cast<unsigned short*>(smem + L::kBeforeAt);
+        unsigned short* list = reinterpret_cast<unsigned short*>(smem + L::kListAt);
+        for (int t = lane_id(); t < L::kWords; t += 32) before[t] = 0;
+        for (int t = lane_id(); t < L::kS; t += 32) list[t] = 0;
+    }
     __syncwarp();
     return smem;
 }
@@ -294,8 +312,9 @@ __global__ void __launch_bounds__(kMergeWarps * 32)
         const long long got =
             merge_range<IT, V, NUMERIC>(c, parts, cur, end, out, out_end, ciC, vC, smem);
         if (lane == 0) {
-            if constexpr (!NUMERIC) rowcnt[i] = got;
-            else if (out + got != out_end) atomicExch(err, (int)kDevCountMismatch);
+            if (got < 0) atomicExch(err, (int)kDevBadIndex);
+            if constexpr (!NUMERIC) rowcnt[i] = max(0LL, got);
+            else if (got >= 0 && out + got != out_end) atomicExch(err, (int)kDevCountMismatch);
         }
     }
 }
@@ -354,6 +373,13 @@ __global__ void __launch_bounds__(kMergeWarps * 32)
         }
         const long long got =
             merge_range<IT, V, NUMERIC>(c, parts, cur, end, out, out_end, ciC, vC, smem);
+        if (got < 0) {   // the row's columns do not ascend
+            if (lane == 0) {
+                atomicExch(err, (int)kDevBadIndex);
+                if constexpr (!NUMERIC) longs->seg[u] = 0;
+            }
+            continue;
+        }
         if (lane == 0) {
             if constexpr (NUMERIC) {
                 if (out + got != out_end || (g + 1 == kMergeSegs && out_end != rpC[i + 1]))
@@ -558,7 +584,7 @@ __global__ void __launch_bounds__(WARPS * 32)
                     long long col = 0;
                     if (valid) {
                         col = (long long)cb[q - bst[s]];
-                        valid = col < c1;
+                        valid = col >= c0 && col < c1;
                     }
                     if (valid) {
                         const int slot = (int)(col - c0);

@@ -136,7 +136,7 @@ spgemm_status spgemm_merge_symbolic_static(int32_t c, const spgemm_csr* parts,
         e = cudaMemcpyAsync(&herr, &cnt->err, sizeof(int), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return static_fail(SPGEMM_ERR_CUDA, cudaGetErrorString(e));
-    if (herr) return static_fail(SPGEMM_ERR_INTERNAL, "device check failed in the merge count");
+    if (herr) return sg::merge_failed(herr);
     *nnz_c = total;
     return SPGEMM_OK;
 }

@@ -110,6 +110,7 @@ spgemm_status check_ws(spgemm_plan_t P, void* ws, size_t ws_bytes);
 // types, semiring); *vt_out = the value kind the merge kernels use.
 spgemm_status check_merge_parts(int32_t c, const spgemm_csr* parts, const spgemm_opts* opts,
                                 int* vt_out);
+spgemm_status merge_failed(int herr);
 cudaError_t run_numeric(Plan* P, unsigned char* w, const int64_t* rowptrC, long long cap,
                         void* colC, void* valC);
 

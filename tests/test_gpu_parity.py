@@ -626,3 +626,58 @@ def test_rows_of_129_to_512_products_sorted(sg, n, value):
         assert_values_close(C, R, A, B, "f32")
     elif value != "none":
         assert np.array_equal(C.to_host()[2], R.val)
+
+
+@pytest.mark.parametrize("c", [1, 2, 4])
+@pytest.mark.parametrize("value", ["u01_f64", "none"])
+@pytest.mark.parametrize("index", [np.int32, np.int64])
+def test_merge_of_rows_that_do_not_ascend(sg, c, value, index):
+    """A part with a row of one repeated column or of descending columns (short,
+    and long enough to be cut into segments), which no chunk can take in
+    order: counts and numeric pass end and report it.  Rows with a column below
+    the chunk's first or after one beyond its span give a sum of some kind.
+    Other rows of the same merge are not disturbed."""
+    import torch
+
+    n = 100_000
+    sr = 1 if value == "none" else 0
+    good = np.arange(0, n, 97)
+    for bad, found in (([5] * 3000, True), (list(range(6000, 0, -1)), True),
+                       (list(range(9000, 0, -1)) + [7] * 3000, True),
+                       ([3, 40_000, 5], False), ([100] + [3] * 40 + list(range(200, 900)), False),
+                       ([9, 2, 60_000, 1] * 200, False)):
+        rng = np.random.default_rng(c)
+        parts = []
+        for s in range(c):
+            rows = [good, np.array(bad if s == c - 1 else good), good]
+            rp = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
+            col = np.concatenate(rows).astype(index)
+            parts.append(sg.to_device(inputs.CSR(3, n, rp, col,
+                                                 inputs.draw_values(rng, col.size, value))))
+        ws = sg.merge_workspace(c, 3, n, "cuda")
+        for count in (lambda: sg.merge_symbolic(parts, ws, sr),
+                      lambda: sg.merge_symbolic_static(parts, sr)):
+            try:
+                count()
+                assert not found
+            except sg.SpgemmError as e:
+                assert e.status == 2        # INVALID_CSR
+        # the numeric pass with row pointers that leave room for every entry
+        ws.zero_()
+        room = good.size + len(bad)
+        rp = torch.tensor([0, good.size, good.size + room, 2 * good.size + room], device="cuda")
+        col = torch.zeros(int(rp[3]), dtype=parts[0].col.dtype, device="cuda")
+        val = None if sr else torch.zeros(int(rp[3]), dtype=torch.float64, device="cuda")
+        sg.merge_numeric(parts, ws, rp, col, val, sr)
+        try:
+            sg.merge_check(ws)
+            assert not found
+        except sg.SpgemmError as e:
+            assert e.status in (2, 8)       # or the bad row's count differs
+        col = col.cpu().numpy()
+        assert np.array_equal(col[:good.size], good) and np.array_equal(col[-good.size:], good)
+        if not sr:
+            want = np.sum([p.val.cpu().numpy()[:good.size] for p in parts], axis=0)
+            got = val.cpu().numpy()[:good.size]
+            # c - 1 additions, each rounded to at most 2^-53 of a sum below c
+            assert np.all(np.abs(got - want) <= c * c * 2.0 ** -53)
