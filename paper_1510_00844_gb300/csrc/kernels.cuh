@@ -2168,72 +2168,94 @@ struct __align__(16) DenseCursor {
 // nextrun[run_base + q] = {length, first column} of the run after it ({0,
 // INT_MAX} at the row's end), so a cursor advances with one load whose address
 // it knows before the chunk's products are accumulated.  Other positions are not
-// written: a cursor only ever stands at the start of a run.  Warp w of WARPS
-// takes every WARPS-th window of 32 entries of the row; the run that leaves a
-// window is followed by a search.  (With a warp per row, window after window
-// from the row's end, and both tables at every entry, the longest rows alone
-// took most of the 613 us of an R-MAT 18 square; now 218 us.)
-template <class IT, int WARPS>
-__device__ __forceinline__ void run_tables_row(const IT* __restrict__ ci, long long s0,
-                                               long long s1, int cw_log2, int32_t* rl, int2* nr,
-                                               int w) {
+// written: a cursor only ever stands at the start of a run.
+
+// A run, as the entries before it need it: its chunk (-1: none, the row's end),
+// its first column, where it ends, and the run after it.  Places count from the
+// row's start.
+struct RunAhead {
+    int chunk, col, end;
+    int2 next;
+};
+
+// The end of the run that place q of the row is in, by the whole warp.
+template <class IT>
+__device__ __forceinline__ int run_end(const IT* __restrict__ ci, int q, int len, int cw_log2) {
+    const int ch = (int)(ci[q] >> cw_log2);
+    int lo = q + 1, hi = len;   // the end is in [lo, hi]
+    while (hi - lo > 32) {
+        const int step = (hi - lo + 31) / 32;
+        const int p = lo + (lane_id() + 1) * step - 1;
+        const unsigned in = __ballot_sync(kFull, p < hi && (int)(ci[min(p, hi - 1)] >> cw_log2) == ch);
+        const int k = __popc(in);
+        hi = min(hi, lo + (k + 1) * step - 1);
+        lo += k * step;
+    }
+    const int p = lo + lane_id();
+    return lo + __popc(__ballot_sync(kFull, p < hi && (int)(ci[min(p, len - 1)] >> cw_log2) == ch));
+}
+
+// Places [a, b) of a row of `len` entries (ci, rl and nr start at the row), by a
+// warp, from the end backwards: 128 entries per step, all loaded at once, and
+// what a window's last run needs to know of the entries after it is carried from
+// lane 0 of the window before.  Every column is read once and both tables are
+// written from registers.
+template <class IT>
+__device__ __forceinline__ void run_tables_range(const IT* __restrict__ ci, int a, int b, int len,
+                                                 int cw_log2, int32_t* __restrict__ rl,
+                                                 int2* __restrict__ nr) {
     const int lane = lane_id();
-    if (WARPS == 1 && s1 - s0 <= 32) {   // one window: the next run is a lane of it
-        const long long q = s0 + lane;
-        const int col = q < s1 ? (int)ci[q] : 0x7fffffff;
-        const int before = __shfl_up_sync(kFull, col, 1);
-        const bool start = q < s1 && (lane == 0 || before >> cw_log2 != col >> cw_log2);
-        const unsigned later = __ballot_sync(kFull, start) & ~lanemask_le();
-        const int next = later ? __ffs(later) - 1 : (int)(s1 - s0);
-        const int len = next - lane;
-        const int next_len = __shfl_sync(kFull, len, next & 31);
-        const int next_col = __shfl_sync(kFull, col, next & 31);
-        if (start) {
-            rl[q] = len;
-            nr[q] = later ? make_int2(next_len, next_col) : make_int2(0, 0x7fffffff);
-        }
-        return;
+    RunAhead ahead{-1, 0x7fffffff, len, make_int2(0, 0x7fffffff)};
+    if (b < len) {
+        ahead.col = (int)ci[b];
+        ahead.chunk = ahead.col >> cw_log2;
+        ahead.end = run_end(ci, b, len, cw_log2);
+        if (ahead.end < len)
+            ahead.next = make_int2(run_end(ci, ahead.end, len, cw_log2) - ahead.end,
+                                   (int)ci[ahead.end]);
     }
-    // whether q starts a run, from its chunk and the chunk of the entry before it
-    auto starts = [&](long long q, long long& ch) {
-        ch = q < s1 ? (long long)ci[q] >> cw_log2 : -2;
-        long long before = __shfl_up_sync(kFull, ch, 1);
-        if (lane == 0) before = q > s0 && q < s1 ? (long long)ci[q - 1] >> cw_log2 : -1;
-        return q < s1 && before != ch;
-    };
-    for (long long lo = s0 + 32 * w; lo < s1; lo += 32 * WARPS) {
-        const long long q = lo + lane;
-        long long ch;
-        const bool start = starts(q, ch);
-        const unsigned later = __ballot_sync(kFull, start) & ~lanemask_le();
-        if (start) {
-            long long end = q + __ffs(later) - 1 - lane;   // the next start in the window
+    for (int hi = b; hi > a; hi -= 128) {
+        // windows [hi - 32 u - 32, hi - 32 u) of lanes; places below a have no entry
+        int col[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int q = hi - 32 * u - 32 + lane;
+            col[u] = q >= a ? (int)ci[q] : -1;
+        }
+        const int first = hi - 128 > 0 ? (int)ci[hi - 129] : -1;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int lo = hi - 32 * u - 32;
+            if (lo + 32 <= a) break;
+            const int q = lo + lane;
+            const int ch = col[u] >> cw_log2;
+            int before = __shfl_up_sync(kFull, ch, 1);
+            const int left = u < 3 ? __shfl_sync(kFull, col[u < 3 ? u + 1 : 3], 31) : first;
+            if (lane == 0) before = left >> cw_log2;
+            if (q == a) before = a > 0 ? (int)(ci[a - 1] >> cw_log2) : -1;
+            const bool start = q >= a && before != ch;
+            const unsigned later = __ballot_sync(kFull, start) & ~lanemask_le();
+            const int t = __ffs(later) - 1;   // the next start in the window, if any
+            int end = lo + t;
+            if (later == 0u) end = ahead.chunk == ch ? ahead.end : lo + 32;
+            int2 next;
+            next.x = __shfl_sync(kFull, end - q, t & 31);
+            next.y = __shfl_sync(kFull, col[u], t & 31);
             if (later == 0u) {
-                // first entry past the window in another chunk; a run has at
-                // most 2^cw_log2 entries
-                long long p = min(s1, lo + 32), e = min(s1, q + (1LL << cw_log2));
-                if (p < e && (long long)ci[p] >> cw_log2 != ch) e = p;
-                while (p < e) {
-                    const long long mid = (p + e) >> 1;
-                    if ((long long)ci[mid] >> cw_log2 == ch) p = mid + 1;
-                    else e = mid;
-                }
-                end = p;
+                if (ahead.chunk == ch) next = ahead.next;
+                else next = make_int2(ahead.end - end, ahead.col);
             }
-            rl[q] = (int32_t)(end - q);
+            if (start) {
+                rl[q] = end - q;
+                nr[q] = next;
+            }
+            ahead.chunk = __shfl_sync(kFull, ch, 0);
+            ahead.col = __shfl_sync(kFull, col[u], 0);
+            ahead.end = __shfl_sync(kFull, end, 0);
+            ahead.next.x = __shfl_sync(kFull, next.x, 0);
+            ahead.next.y = __shfl_sync(kFull, next.y, 0);
         }
     }
-    if constexpr (WARPS > 1) __syncthreads();   // the row's run lengths are visible
-    else __syncwarp();
-    for (long long lo = s0 + 32 * w; lo < s1; lo += 32 * WARPS) {
-        const long long q = lo + lane;
-        long long ch;
-        if (starts(q, ch)) {
-            const long long q2 = q + rl[q];
-            nr[q] = q2 < s1 ? make_int2(rl[q2], (int)ci[q2]) : make_int2(0, 0x7fffffff);
-        }
-    }
-    __syncwarp();
 }
 
 template <class IT>
@@ -2263,12 +2285,19 @@ __device__ __forceinline__ void runlen_kernel_body(long long LB, const ProdDesc*
     const long long nwarps = ((long long)vnb * blockDim.x) >> 5;
     for (long long kb = warp; kb < LB; kb += nwarps) {
         const BRow<IT> r = b_row<IT>(D, bb, nprod, kb);
-        run_tables_row<IT, 1>(r.ci, r.s0, r.s1, cw_log2, runlen + r.run_base,
-                              nextrun + r.run_base, 0);
+        run_tables_range<IT>(r.ci + r.s0, 0, (int)(r.s1 - r.s0), (int)(r.s1 - r.s0), cw_log2,
+                             runlen + r.run_base + r.s0, nextrun + r.run_base + r.s0);
     }
 }
 
-// A warp per B row, a block for the longest.
+// A warp per B row; eight, each a part of it, for a row of more than kRunLong.
+// What bounds it: instructions and the stores (12 bytes per run).  Two passes
+// per row, windows of 32 loaded one after another and a block for rows of more
+// than 512 entries took, in us: R-MAT, 65536 vertices 83, now 41; scale 18 219
+// and 142; the 0.75 G entries of a Markov step on 2^20 vertices, whose rows of
+// 711 entries have runs of one or two, 10670 and 4390.  The limit: 1024 30, 119
+// and 4750; 4096 41, 143 and 4260.
+constexpr int kRunLong = 2048;
 template <class IT>
 __global__ void __launch_bounds__(32 * kRowWarps)
     runlen_kernel(long long LB, const ProdDesc* __restrict__ D,
@@ -2283,17 +2312,20 @@ __global__ void __launch_bounds__(32 * kRowWarps)
         const long long kb = tile * kRowWarps + w;
         BRow<IT> r{nullptr, 0, 0, 0};
         if (kb < LB) r = b_row<IT>(D, bb, nprod, kb);
-        const bool big = r.s1 - r.s0 > 512;
-        if (!big && r.s1 > r.s0)
-            run_tables_row<IT, 1>(r.ci, r.s0, r.s1, cw_log2, runlen + r.run_base,
-                                  nextrun + r.run_base, 0);
+        const bool big = r.s1 - r.s0 > kRunLong;
+        if (!big)
+            run_tables_range<IT>(r.ci + r.s0, 0, (int)(r.s1 - r.s0), (int)(r.s1 - r.s0), cw_log2,
+                                 runlen + r.run_base + r.s0, nextrun + r.run_base + r.s0);
         if (lane_id() == 0) longs[w] = big ? r : BRow<IT>{nullptr, 0, 0, 0};
         if (__syncthreads_or(big))
             for (int t = 0; t < kRowWarps; ++t) {
                 const BRow<IT> x = longs[t];
-                if (x.s1 > x.s0)
-                    run_tables_row<IT, kRowWarps>(x.ci, x.s0, x.s1, cw_log2, runlen + x.run_base,
-                                                  nextrun + x.run_base, w);
+                const int len = (int)(x.s1 - x.s0);
+                const int per = ((len + kRowWarps - 1) / kRowWarps + 127) & ~127;
+                const int from = min(len, per * w), to = min(len, from + per);
+                if (from < to)
+                    run_tables_range<IT>(x.ci + x.s0, from, to, len, cw_log2,
+                                         runlen + x.run_base + x.s0, nextrun + x.run_base + x.s0);
             }
         __syncthreads();   // the list has been read
     }

@@ -681,3 +681,40 @@ def test_merge_of_rows_that_do_not_ascend(sg, c, value, index):
             got = val.cpu().numpy()[:good.size]
             # c - 1 additions, each rounded to at most 2^-53 of a sum below c
             assert np.all(np.abs(got - want) <= c * c * 2.0 ** -53)
+
+
+@pytest.mark.parametrize("n", [3000, 200_000, 1_800_000])
+@pytest.mark.parametrize("index", [np.int32, np.int64])
+def test_dense_rows_over_runs_of_every_kind(sg, n, index):
+    """The run tables of B on rows at the edges of a warp's window (32 entries), of
+    its step (128) and of the rows that several warps share (beyond 2048): runs
+    of one or a few entries, one run over many windows, and both in turn; rows of
+    A that are dense over them."""
+    rng = np.random.default_rng(n % 997)
+    lens = [0, 1, 2, 31, 32, 33, 64, 65, 127, 128, 129, 160, 161, 1023, 1024, 1025, 2047, 2048,
+            2049, 2176, 2177, 2900, 5000, 20_000]
+    cols = []
+    for k in lens:
+        if k > n:
+            continue
+        cols.append(rng.choice(n, k, replace=False))                       # spread
+        cols.append(np.arange(k))                                          # side by side
+        cols.append(n - k + np.arange(k))
+        step = max(1, min(n // max(k, 1), 1500))
+        cols.append(np.arange(k) * step)                                   # evenly
+        half = np.concatenate([np.arange(k // 2), n - 1 - 40 * np.arange(k - k // 2)])
+        cols.append(np.unique(np.clip(half, 0, n - 1)))                    # a block, then apart
+    cols = [np.sort(c) for c in cols]
+    size = np.array([c.size for c in cols])
+    B = inputs.CSR(len(cols), n, np.concatenate([[0], np.cumsum(size)]).astype(np.int64),
+                   np.concatenate(cols).astype(index), rng.random(int(size.sum())))
+    rows = [np.sort(rng.choice(len(cols), k, replace=False)) for k in (1, 5, 20, 40, 60, 90)
+            for _ in range(4)] + [np.arange(len(cols))]
+    rows += [np.array([t]) for t in range(len(cols))]
+    colA = np.concatenate(rows).astype(index)
+    rpA = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
+    A = inputs.CSR(len(rows), len(cols), rpA, colA, rng.random(colA.size))
+    C = run(sg, A, B)
+    R = oracle.spgemm(A, B)
+    assert_pattern_equal(C, R)
+    assert np.array_equal(C.to_host()[2], R.val)
