@@ -331,7 +331,17 @@ cudaError_t launch_chain(const ChainProduct* steps, ChainSync* sync, int max_wor
             sym_groups = gg;
             break;
         }
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit belongs to the kernel, so it is the device's whatever this chain's
+    // size is: a chain of another thread must not find a smaller one
+    cudaFuncAttributes attr;
+    int dev = 0, most = 0;
+    cudaError_t e = cudaFuncGetAttributes(&attr, k);
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 std::max((int)smem, most - (int)attr.sharedSizeBytes));
     if (e != cudaSuccess) return e;
     int occ = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, THREADS, smem);

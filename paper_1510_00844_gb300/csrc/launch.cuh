@@ -17,10 +17,18 @@ int occupancy_blocks(F kernel, int threads, size_t smem) {
     return occupancy_lookup(reinterpret_cast<const void*>(kernel), threads, smem);
 }
 
+// Lets a launch of `kernel` take `smem` bytes of shared memory.  The limit belongs
+// to the kernel, not to the launch, so where sizes differ from call to call it is
+// set to `most`, the largest of them: another thread's launch between this call
+// and its own finds the same limit, never a smaller one.
 template <class F>
-cudaError_t allow_smem(F kernel, size_t smem) {
+cudaError_t allow_smem(F kernel, size_t smem, size_t most) {
     if (smem <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+template <class F>
+cudaError_t allow_smem(F kernel, size_t smem) {   // the kernel's only size
+    return allow_smem(kernel, smem, smem);
 }
 
 inline long long grid_for(long long work_items, int per_block, int sm_count, int occ) {
@@ -112,7 +120,7 @@ template <class IT>
 cudaError_t sym_rank_bin(Plan& P, int bin, long long nrows, int64_t* rowcnt) {
     auto k = symbolic_rank_kernel<IT>;
     const size_t smem = RankSmem<NoVal>(P.max_n, true).total;
-    cudaError_t e = allow_smem(k, smem);
+    cudaError_t e = allow_smem(k, smem, RankSmem<NoVal>(rank_max_n(3, true), true).total);
     if (e != cudaSuccess) return e;
     const int occ = occupancy_blocks(k, 32 * kRankWarps, smem);
     count_launches(1);
@@ -127,7 +135,7 @@ cudaError_t num_rank_bin(Plan& P, int bin, long long nrows, const int64_t* rpC, 
                          unsigned* overflow_count) {
     auto k = numeric_rank_kernel<IT, V>;
     const size_t smem = RankSmem<V>(P.max_n, false).total;
-    cudaError_t e = allow_smem(k, smem);
+    cudaError_t e = allow_smem(k, smem, RankSmem<V>(rank_max_n(3, false), false).total);
     if (e != cudaSuccess) return e;
     const int occ = occupancy_blocks(k, 32 * kRankWarps, smem);
     count_launches(1);
@@ -226,8 +234,9 @@ cudaError_t launch_symbolic(Plan& P, unsigned char* ws, int64_t* rowcnt) {
         auto kb = symbolic_dense_kernel<IT, 1024, 1>;
         const int max_words = (int)((std::min(P.max_n, P.max_dense_n) + 31) / 32);
         size_t smem = (size_t)max_words * 4;
-        if ((e = allow_smem(ks, smem)) != cudaSuccess) return e;
-        if ((e = allow_smem(kb, smem)) != cudaSuccess) return e;
+        const size_t most = (size_t)((P.max_dense_n + 31) / 32) * 4;
+        if ((e = allow_smem(ks, smem, most)) != cudaSuccess) return e;
+        if ((e = allow_smem(kb, smem, most)) != cudaSuccess) return e;
         int threads = 256, occ = occupancy_blocks(ks, 256, smem);
         const int o512 = occupancy_blocks(ks, 512, smem);
         if (o512 * 512 > occ * threads) { threads = 512; occ = o512; }

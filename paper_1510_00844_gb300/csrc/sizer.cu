@@ -16,6 +16,7 @@
 namespace sg {
 
 constexpr int kSizerH = 32;
+constexpr int kSizerMostF = 64;
 constexpr int kSizerTile = 128;
 
 __host__ __device__ constexpr int sizer_params(int F) {
@@ -170,8 +171,11 @@ cudaError_t launch_sizer_grad(const float* X, const float* T, const long long* o
                               long long s0, long long count, int F, float norm, const float* prm,
                               float* grad, float* loss, cudaStream_t s, int sms) {
     const size_t smem = grad_smem(F);
+    // the limit belongs to the kernel: the same for every F, so that threads with
+    // different ones do not lower each other's
     cudaError_t e = cudaFuncSetAttribute(sizer_grad_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)grad_smem(kSizerMostF));
     if (e != cudaSuccess) return e;
     const long long tiles = (count + kSizerTile - 1) / kSizerTile;
     const unsigned g = (unsigned)std::max<long long>(1, std::min<long long>(tiles, (long long)sms * 2));
@@ -219,7 +223,7 @@ int32_t spgemm_sizer_param_count(int32_t features) { return sg::sizer_params(fea
 
 spgemm_status spgemm_sizer_forward(const float* X, int64_t N, int32_t F, const float* params,
                                    float* y, void* stream) {
-    if (N < 0 || F < 1 || F > 64 || (N > 0 && (!X || !params || !y))) {
+    if (N < 0 || F < 1 || F > sg::kSizerMostF || (N > 0 && (!X || !params || !y))) {
         sg::set_last_error("sizer_forward: bad arguments");
         return SPGEMM_ERR_INVALID_ARG;
     }
@@ -241,7 +245,7 @@ spgemm_status spgemm_sizer_forward(const float* X, int64_t N, int32_t F, const f
 
 spgemm_status spgemm_sizer_grad(const float* X, const float* T, int64_t N, int32_t F,
                                 const float* params, float* grad, float* loss, void* stream) {
-    if (N <= 0 || F < 1 || F > 64 || !X || !T || !params || !grad || !loss) {
+    if (N <= 0 || F < 1 || F > sg::kSizerMostF || !X || !T || !params || !grad || !loss) {
         sg::set_last_error("sizer_grad: bad arguments");
         return SPGEMM_ERR_INVALID_ARG;
     }
@@ -264,7 +268,7 @@ spgemm_status spgemm_sizer_train(const float* X, const float* T, const int64_t* 
                                  int32_t F, float* params, float* adam_m, float* adam_v,
                                  float* grad, int32_t steps, int32_t batch, float lr,
                                  float* loss_trace, void* stream) {
-    if (N <= 0 || F < 1 || F > 64 || steps < 0 || batch < 1 || !X || !T || !order || !params ||
+    if (N <= 0 || F < 1 || F > sg::kSizerMostF || steps < 0 || batch < 1 || !X || !T || !order || !params ||
         !adam_m || !adam_v || !grad || !loss_trace) {
         sg::set_last_error("sizer_train: bad arguments");
         return SPGEMM_ERR_INVALID_ARG;
@@ -318,7 +322,7 @@ spgemm_status spgemm_sizer_targets(const int64_t* rowptrC, int64_t m, float* T, 
 
 spgemm_status spgemm_sizer_save(const float* params, int32_t F, void* stream, void* buf,
                                 size_t buf_bytes, size_t* bytes_out) {
-    if (F < 1 || F > 64 || !bytes_out) {
+    if (F < 1 || F > sg::kSizerMostF || !bytes_out) {
         sg::set_last_error("sizer_save: bad arguments");
         return SPGEMM_ERR_INVALID_ARG;
     }
@@ -351,7 +355,7 @@ spgemm_status spgemm_sizer_save(const float* params, int32_t F, void* stream, vo
 spgemm_status spgemm_sizer_load(const void* buf, size_t buf_bytes, int32_t F, float* params,
                                 void* stream) {
     const unsigned char* in = (const unsigned char*)buf;
-    if (!in || F < 1 || F > 64) {
+    if (!in || F < 1 || F > sg::kSizerMostF) {
         sg::set_last_error("sizer_load: bad arguments");
         return SPGEMM_ERR_INVALID_ARG;
     }

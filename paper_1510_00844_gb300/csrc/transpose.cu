@@ -358,8 +358,11 @@ cudaError_t launch_transpose(const spgemm_csr& A, cudaStream_t s, unsigned char*
         const size_t bitmap = sizeof(uint2) * (size_t)std::min<long long>(kTrWords, (m + 31) / 32);
         // a row that takes the bitonic sort has m > kTrBitsPerEntry * kTrWarpMax
         const size_t smem = m > (long long)kTrBitsPerEntry * kTrWarpMax ? std::max(bitonic, bitmap) : bitmap;
+        // the limit belongs to the kernel: a call of another height, in another
+        // thread, must find the same one
+        const size_t most = std::max(bitonic, sizeof(uint2) * (size_t)kTrWords);
         if (smem > 48 * 1024 &&
-            (e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+            (e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most)) != cudaSuccess)
             return e;
         k<<<blocks(std::min<long long>(n, nnz / kTrWarpMax + 1), 1, smem > 74 * 1024 ? 2 : 3), THREADS, smem, s>>>(
             long_rows, long_count, m, rpT, ciS, vaS, ciT, vaT);
