@@ -2226,7 +2226,6 @@ __device__ __forceinline__ void run_tables_range(const IT* __restrict__ ci, int 
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const int lo = hi - 32 * u - 32;
-            if (lo + 32 <= a) break;
             const int q = lo + lane;
             const int ch = col[u] >> cw_log2;
             int before = __shfl_up_sync(kFull, ch, 1);
@@ -2249,12 +2248,36 @@ __device__ __forceinline__ void run_tables_range(const IT* __restrict__ ci, int 
                 rl[q] = end - q;
                 nr[q] = next;
             }
+            if (lo <= a) break;
             ahead.chunk = __shfl_sync(kFull, ch, 0);
             ahead.col = __shfl_sync(kFull, col[u], 0);
             ahead.end = __shfl_sync(kFull, end, 0);
             ahead.next.x = __shfl_sync(kFull, next.x, 0);
             ahead.next.y = __shfl_sync(kFull, next.y, 0);
         }
+    }
+}
+
+// A whole row, by a warp.  Rows of at most 32 entries are one window and need no
+// carry.
+template <class IT>
+__device__ __forceinline__ void run_tables_row(const IT* __restrict__ ci, int len, int cw_log2,
+                                               int32_t* __restrict__ rl, int2* __restrict__ nr) {
+    if (len > 32) {
+        run_tables_range<IT>(ci, 0, len, len, cw_log2, rl, nr);
+        return;
+    }
+    const int q = lane_id();
+    const int col = q < len ? (int)ci[q] : 0x7fffffff;
+    const int before = __shfl_up_sync(kFull, col, 1);
+    const bool start = q < len && (q == 0 || before >> cw_log2 != col >> cw_log2);
+    const unsigned later = __ballot_sync(kFull, start) & ~lanemask_le();
+    const int next = later ? __ffs(later) - 1 : len;
+    const int next_len = __shfl_sync(kFull, next - q, next & 31);
+    const int next_col = __shfl_sync(kFull, col, next & 31);
+    if (start) {
+        rl[q] = next - q;
+        nr[q] = later ? make_int2(next_len, next_col) : make_int2(0, 0x7fffffff);
     }
 }
 
@@ -2285,21 +2308,23 @@ __device__ __forceinline__ void runlen_kernel_body(long long LB, const ProdDesc*
     const long long nwarps = ((long long)vnb * blockDim.x) >> 5;
     for (long long kb = warp; kb < LB; kb += nwarps) {
         const BRow<IT> r = b_row<IT>(D, bb, nprod, kb);
-        run_tables_range<IT>(r.ci + r.s0, 0, (int)(r.s1 - r.s0), (int)(r.s1 - r.s0), cw_log2,
-                             runlen + r.run_base + r.s0, nextrun + r.run_base + r.s0);
+        run_tables_row<IT>(r.ci + r.s0, (int)(r.s1 - r.s0), cw_log2, runlen + r.run_base + r.s0,
+                           nextrun + r.run_base + r.s0);
     }
 }
 
 // A warp per B row; eight, each a part of it, for a row of more than kRunLong.
 // What bounds it: instructions and the stores (12 bytes per run).  Two passes
 // per row, windows of 32 loaded one after another and a block for rows of more
-// than 512 entries took, in us: R-MAT, 65536 vertices 83, now 41; scale 18 219
-// and 142; the 0.75 G entries of a Markov step on 2^20 vertices, whose rows of
-// 711 entries have runs of one or two, 10670 and 4390.  The limit: 1024 30, 119
-// and 4750; 4096 41, 143 and 4260.
+// than 512 entries took, in us: R-MAT, 65536 vertices 83, now 35; scale 18 218
+// and 123; the 0.75 G entries of a Markov step on 2^20 vertices, whose rows of
+// 711 entries have runs of one or two, 10670 and 3610.  The limit, before the
+// register cap: 1024 30, 119 and 4750; 2048 41, 142 and 4390; 4096 41, 143 and
+// 4260.  The cap keeps six blocks resident (five without: 36, 129 and 3750; eight
+// spill: 45, 141 and 3520).
 constexpr int kRunLong = 2048;
 template <class IT>
-__global__ void __launch_bounds__(32 * kRowWarps)
+__global__ void __launch_bounds__(32 * kRowWarps, 6)
     runlen_kernel(long long LB, const ProdDesc* __restrict__ D,
                   const long long* __restrict__ bb, int nprod, int cw_log2,
                   int32_t* __restrict__ runlen, int2* __restrict__ nextrun,
@@ -2313,9 +2338,9 @@ __global__ void __launch_bounds__(32 * kRowWarps)
         BRow<IT> r{nullptr, 0, 0, 0};
         if (kb < LB) r = b_row<IT>(D, bb, nprod, kb);
         const bool big = r.s1 - r.s0 > kRunLong;
-        if (!big)
-            run_tables_range<IT>(r.ci + r.s0, 0, (int)(r.s1 - r.s0), (int)(r.s1 - r.s0), cw_log2,
-                                 runlen + r.run_base + r.s0, nextrun + r.run_base + r.s0);
+        if (!big && r.s1 > r.s0)
+            run_tables_row<IT>(r.ci + r.s0, (int)(r.s1 - r.s0), cw_log2, runlen + r.run_base + r.s0,
+                               nextrun + r.run_base + r.s0);
         if (lane_id() == 0) longs[w] = big ? r : BRow<IT>{nullptr, 0, 0, 0};
         if (__syncthreads_or(big))
             for (int t = 0; t < kRowWarps; ++t) {

@@ -204,9 +204,11 @@ cudaError_t launch_dense_tables(Plan& P, unsigned char* ws) {
         segtab_kernel<IT><<<(unsigned)g, 256, 0, P.stream>>>(P.LB, P.d_descs, P.bb, P.nprod, P.cw_log2,
                                                              (int32_t*)(ws + L.segtab), P.cnt);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        long long g2 = grid_for(P.LB, 8, P.sm_count, 8);
+        auto k = runlen_kernel<IT>;
+        const long long g2 =
+            grid_for(P.LB, kRowWarps, P.sm_count, occupancy_blocks(k, 32 * kRowWarps, 0));
         count_launches(1);
-        runlen_kernel<IT><<<(unsigned)g2, 256, 0, P.stream>>>(P.LB, P.d_descs, P.bb, P.nprod, P.cw_log2,
+        k<<<(unsigned)g2, 256, 0, P.stream>>>(P.LB, P.d_descs, P.bb, P.nprod, P.cw_log2,
                                                               (int32_t*)(ws + L.runlen),
                                                               (int2*)(ws + L.nextrun), P.cnt);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
