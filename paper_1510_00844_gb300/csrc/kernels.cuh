@@ -1115,7 +1115,7 @@ __global__ void __launch_bounds__(MAXT, MINB) symbolic_dense_kernel(const ProdDe
 // and a scan for each 0.63 ms, four 0.59 ms; loading a step ahead 0.60 ms.
 constexpr int kColStage = 512;   // of the 4096 columns of 128 words
 template <class IT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 8)
     dense_columns_kernel(const ProdDesc* __restrict__ D, const long long* __restrict__ rb,
                          int nprod, const int32_t* __restrict__ rows, const DevCounters* cnt,
                          const unsigned* __restrict__ kept, int max_words, int chunk_words,
@@ -1141,7 +1141,9 @@ __global__ void __launch_bounds__(256)
         }
         before = warp_sum(before);
         own = warp_sum(own);
-        if (end > cap || (w == 7 && out + before + own != end)) {
+        // the row pointers are the caller's: no warp writes outside its part of them
+        if (out < 0 || end > cap || out + before + own > end ||
+            (w == 7 && out + before + own != end)) {
             if (lane == 0) atomicExch(err, end > cap ? (int)kDevCapacity : (int)kDevCountMismatch);
             continue;
         }

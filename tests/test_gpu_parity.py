@@ -718,3 +718,31 @@ def test_dense_rows_over_runs_of_every_kind(sg, n, index):
     R = oracle.spgemm(A, B)
     assert_pattern_equal(C, R)
     assert np.array_equal(C.to_host()[2], R.val)
+
+
+def test_pattern_with_row_pointers_of_another_product(sg):
+    """Row pointers that are not the plan's: every row short and at the end of the
+    arrays, in front of them, or beyond them.  Reported, and nothing is written
+    outside the columns handed over."""
+    import torch
+
+    n, l = 40_000, 60
+    A = inputs.random_csr(30, l, 0.9, 71, value="none", index_dtype=np.int32)
+    B = inputs.random_csr(l, n, 0.05, 72, value="none", index_dtype=np.int32)
+    p = sg.plan(sg.to_device(A), sg.to_device(B), semiring=1)
+    assert p.info()["rows_dense"] == 30
+    rp, nnz = sg.symbolic(p)
+    room = torch.full((nnz + 2 * n,), -7, dtype=torch.int32, device="cuda")
+    col = room[n:n + nnz]
+    base = torch.arange(31, device="cuda")
+    for other in (torch.full_like(rp, nnz), nnz - 30 + base, base - 15, rp + 1, rp.flip(0)):
+        sg.numeric(p, other.to(torch.int64).contiguous(), col, None)
+        with pytest.raises(sg.SpgemmError):
+            sg.check(p)
+        assert bool((room[:n] == -7).all()) and bool((room[n + nnz:] == -7).all())
+        p = sg.plan(sg.to_device(A), sg.to_device(B), semiring=1)
+        rp, nnz = sg.symbolic(p)
+    sg.numeric(p, rp, col, None)
+    sg.check(p)
+    R = oracle.spgemm(A, B, semiring="or_and")
+    assert np.array_equal(col.cpu().numpy().astype(np.int64), R.col)
