@@ -356,11 +356,17 @@ spgemm_status spgemm_learned_multiply(const spgemm_csr* A, const spgemm_csr* B,
 /* Statistics of a plan (host call, no device work). */
 spgemm_status spgemm_plan_info(spgemm_plan_t plan, spgemm_info* info);
 
-/* Device workspace (bytes) that spgemm_symbolic / spgemm_numeric need for
- * this plan (dense-chunk counts and per-entry cursors; for OR_AND also a
- * bitmap of n bits per dense row while all of them take at most a byte per
- * product and 8 GB).  Host call. */
+/* Device workspace (bytes) that spgemm_symbolic / spgemm_numeric use for
+ * this plan (dense-chunk counts and per-entry cursors; for OR_AND, in place of
+ * the cursors, a bitmap of n bits per dense row while all of them take at most a
+ * byte per product and 8 GB).  Host call. */
 spgemm_status spgemm_workspace_size(spgemm_plan_t plan, size_t* bytes);
+
+/* The least workspace they accept: that without the bitmaps, where it is the
+ * smaller one.  With fewer bytes than spgemm_workspace_size the products of an
+ * OR_AND plan's dense rows are gone through a second time (same result).  The
+ * workspace that spgemm_symbolic got is the one for spgemm_numeric.  Host call. */
+spgemm_status spgemm_workspace_least(spgemm_plan_t plan, size_t* bytes);
 
 /* spgemm_symbolic -- count the nonzeros of every row of C (the size of the
  * union of the column sets of the rows of B selected by A(i,:)), write the

@@ -106,17 +106,17 @@ static std::atomic<long long> g_launches{0};
 void count_launches(long long k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 void set_last_error(const char* msg) { g_last_error = msg; }
 
-WsLayout workspace_layout(const Plan& P) {
+WsLayout workspace_layout(const Plan& P, bool keep_bits) {
     WsLayout L;
     const bool dense = P.device_sized || P.ndense > 0;
     size_t off = 0;
     L.chunkcnt = off;
     if (dense) off += align_up((size_t)P.chunk_total * sizeof(int32_t));
     L.kept = off;
-    if (P.keep_bits)
+    if (keep_bits)
         off += align_up((size_t)P.ndense * ((std::min(P.max_n, P.max_dense_n) + 31) / 32) *
                         sizeof(unsigned));
-    const bool tables = dense && !P.keep_bits;   // what the sweep over the products needs
+    const bool tables = dense && !keep_bits;   // what the sweep over the products needs
     L.segtab = off;
     if (tables) off += align_up((size_t)P.seg_total * sizeof(int32_t));
     L.runlen = off;
@@ -381,10 +381,13 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
     {
         // A pattern's dense rows are in the bitmaps of the symbolic pass: they
         // are kept while they take no more than a byte per product (the columns
-        // of C take up to four) and 8 GB.  Learned plans have no symbolic pass.
+        // of C take up to four) and 8 GB, and while the caller's workspace has
+        // room for them (else the products are swept again).  Learned plans have no
+        // symbolic pass.
         const double bytes = (double)P->ndense * (double)std::min(P->max_n, P->max_dense_n) / 8;
-        P->keep_bits = vt == SPGEMM_BOOL && !P->prm && P->ndense > 0 &&
-                       bytes <= (double)P->total_flops && bytes <= 8e9;
+        P->may_keep_bits = vt == SPGEMM_BOOL && !P->prm && P->ndense > 0 &&
+                           bytes <= (double)P->total_flops && bytes <= 8e9;
+        P->keep_bits = P->may_keep_bits;
     }
     if (!o.seg_log2 && P->ndense > 0) {
         // dense work units of about total_flops / (4 x resident dense warps)
@@ -546,7 +549,14 @@ spgemm_status spgemm_plan_info(spgemm_plan_t P, spgemm_info* info) {
 
 spgemm_status spgemm_workspace_size(spgemm_plan_t P, size_t* bytes) {
     if (!P || !bytes) return fail(SPGEMM_ERR_INVALID_ARG, "NULL argument");
-    *bytes = sg::workspace_layout(*P).total;
+    *bytes = sg::workspace_layout(*P, P->may_keep_bits).total;
+    return SPGEMM_OK;
+}
+
+spgemm_status spgemm_workspace_least(spgemm_plan_t P, size_t* bytes) {
+    if (!P || !bytes) return fail(SPGEMM_ERR_INVALID_ARG, "NULL argument");
+    *bytes = std::min(sg::workspace_layout(*P, P->may_keep_bits).total,
+                      sg::workspace_layout(*P, false).total);
     return SPGEMM_OK;
 }
 
@@ -556,6 +566,11 @@ spgemm_status spgemm_symbolic(spgemm_plan_t P, void* ws, size_t ws_bytes, int64_
     if (!P || !rowptrC || !nnz_c) return fail(SPGEMM_ERR_INVALID_ARG, "NULL argument");
     if (P->device_sized)
         return fail(SPGEMM_ERR_INVALID_ARG, "device-sized plans run through spgemm_execute");
+    // the bitmaps of a pattern's dense rows are kept if there is room for them, or
+    // if the tables of the sweep would need more
+    P->keep_bits = P->may_keep_bits;
+    if (P->keep_bits && ws_bytes < sg::workspace_layout(*P).total)
+        P->keep_bits = sg::workspace_layout(*P).total <= sg::workspace_layout(*P, false).total;
     spgemm_status st = check_ws(P, ws, ws_bytes);
     if (st != SPGEMM_OK) return st;
     cudaStream_t s = P->stream;

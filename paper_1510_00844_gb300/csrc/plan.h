@@ -31,7 +31,8 @@ struct spgemm_plan_s {
     int hash_shift = 0;      // hash rows are binned by flops << hash_shift
     int seg_log2 = 16;       // dense work units of about 2^seg_log2 products
     bool device_sized = false;  // no host readback: sizes are upper bounds
-    bool keep_bits = false;  // pattern only: the symbolic pass keeps the dense rows' bitmaps
+    bool may_keep_bits = false;  // pattern only: the symbolic pass may keep the dense rows' bitmaps
+    bool keep_bits = false;      // ... and does: the last symbolic workspace had room for them
     // plan workspace
     unsigned char* pws = nullptr;
     size_t pws_bytes = 0;
@@ -98,7 +99,8 @@ struct WsLayout {
     size_t chunkcnt = 0, kept = 0, segtab = 0, runlen = 0, nextrun = 0, arena = 0, scan = 0, total = 0;
     long long arena_stride = 0;
 };
-WsLayout workspace_layout(const Plan& P);
+WsLayout workspace_layout(const Plan& P, bool keep_bits);
+inline WsLayout workspace_layout(const Plan& P) { return workspace_layout(P, P.keep_bits); }
 size_t plan_workspace_bytes(int nprod, long long R);
 
 spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,

@@ -116,6 +116,7 @@ def _load():
         "spgemm_transpose": (st, [P, P, P, S, P, P, P]),
         "spgemm_plan_info": (st, [P, P]),
         "spgemm_workspace_size": (st, [P, P]),
+        "spgemm_workspace_least": (st, [P, P]),
         "spgemm_symbolic": (st, [P, P, S, P, P]),
         "spgemm_numeric": (st, [P, P, S, P, P, P]),
         "spgemm_check": (st, [P]),
@@ -245,9 +246,27 @@ class Plan:
                                 ctypes.c_void_p(self._plan_ws.data_ptr()),
                                 self._plan_ws.numel(), ctypes.byref(h)))
         self._h = h
+        self._alloc_workspace()
+
+    def _alloc_workspace(self, least: bool = False):
+        """The workspace of spgemm_workspace_size, or that of
+        spgemm_workspace_least where the device has no room for it."""
         nb = ctypes.c_size_t()
-        _check(_lib.spgemm_workspace_size(self._h, ctypes.byref(nb)))
-        self.ws = _workspace(nb.value, self.device)
+        if not least:
+            _check(_lib.spgemm_workspace_size(self._h, ctypes.byref(nb)))
+            try:
+                self.ws = _workspace(nb.value, self.device)
+                return
+            except torch.OutOfMemoryError:
+                if nb.value == self.least_workspace():
+                    raise
+        self.ws = None
+        self.ws = _workspace(self.least_workspace(), self.device)
+
+    def least_workspace(self) -> int:
+        nb = ctypes.c_size_t()
+        _check(_lib.spgemm_workspace_least(self._h, ctypes.byref(nb)))
+        return nb.value
 
     def info(self) -> dict:
         inf = _Info()
@@ -301,9 +320,7 @@ class BatchPlan(Plan):
                   ctypes.c_void_p(self._plan_ws.data_ptr()), self._plan_ws.numel(),
                   ctypes.byref(h)))
         self._h = h
-        nb = ctypes.c_size_t()
-        _check(_lib.spgemm_workspace_size(self._h, ctypes.byref(nb)))
-        self.ws = _workspace(nb.value, self.device)
+        self._alloc_workspace()
 
 
 def batch_plan(As, Bs, semiring: int = PLUS_TIMES, checked: bool = False, stream=None,
@@ -470,10 +487,24 @@ def check(p: Plan) -> None:
     _check(_lib.spgemm_check(p._h))
 
 
-def alloc_output(p: Plan, nnz: int):
+def _output(p: Plan, nnz: int):
     colC = torch.empty(nnz, dtype=p.A.col.dtype, device=p.device)
     valC = None if p.pattern_only else torch.empty(nnz, dtype=p.A.val.dtype, device=p.device)
     return colC, valC
+
+
+def alloc_output(p: Plan, nnz: int):
+    """Column and value arrays of C.  Where the device has no room for them beside
+    a workspace that could be smaller, it is made so and the counts are
+    repeated in it."""
+    try:
+        return _output(p, nnz)
+    except torch.OutOfMemoryError:
+        if p.ws.numel() <= max(p.least_workspace(), 1):
+            raise
+    p._alloc_workspace(least=True)
+    symbolic(p)
+    return _output(p, nnz)
 
 
 def spgemm(A: DeviceCSR, B: DeviceCSR, semiring: int = PLUS_TIMES, checked: bool = False,

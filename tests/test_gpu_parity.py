@@ -746,3 +746,68 @@ def test_pattern_with_row_pointers_of_another_product(sg):
     sg.check(p)
     R = oracle.spgemm(A, B, semiring="or_and")
     assert np.array_equal(col.cpu().numpy().astype(np.int64), R.col)
+
+
+def test_pattern_without_room_for_bitmaps(sg, monkeypatch):
+    """A pattern plan takes any workspace from spgemm_workspace_least on, with the
+    same result, and falls back to it where the device has no room for its
+    bitmaps or, beside them, for C."""
+    import torch
+
+    n, l = 1_800_000, 30
+    A = inputs.random_csr(60, l, 0.97, 81, value="none", index_dtype=np.int32)
+    rng = np.random.default_rng(82)
+    cols = [np.sort(rng.choice(n, 10_000, replace=False)) for _ in range(l)]
+    B = inputs.CSR(l, n, (np.arange(l + 1) * 10_000).astype(np.int64),
+                   np.concatenate(cols).astype(np.int32), None)
+    dA, dB = sg.to_device(A), sg.to_device(B)
+    R = oracle.spgemm(A, B, semiring="or_and")
+
+    def right(rp, col):
+        return (np.array_equal(rp.cpu().numpy(), R.rowptr)
+                and np.array_equal(col.cpu().numpy().astype(np.int64), R.col))
+
+    p = sg.plan(dA, dB, semiring=1)
+    full, least = p.ws.numel(), p.least_workspace()
+    assert p.info()["rows_dense"] == 60 and least < full
+    for size in (full - 1, least, full, full + 1, least + 1):
+        p.ws = sg._workspace(size, "cuda")
+        rp, nnz = sg.symbolic(p)
+        col, _ = sg.alloc_output(p, nnz)
+        sg.numeric(p, rp, col, None)
+        sg.check(p)
+        assert p.ws.numel() == size and right(rp, col)
+    p.ws = sg._workspace(least - 1, "cuda")
+    with pytest.raises(sg.SpgemmError) as e:
+        sg.symbolic(p)
+    assert e.value.status == 4          # OUT_OF_MEMORY
+
+    # no room for the larger workspace
+    make, sizes = sg._workspace, []
+
+    def small_only(nbytes, device):
+        sizes.append(nbytes)
+        if nbytes >= full:
+            raise torch.OutOfMemoryError("no room")
+        return make(nbytes, device)
+
+    monkeypatch.setattr(sg, "_workspace", small_only)
+    C = sg.spgemm(dA, dB, semiring=1, verify=True)
+    assert full in sizes and sizes[-1] == least and right(C.rowptr, C.col)
+    monkeypatch.setattr(sg, "_workspace", make)
+
+    # no room for C beside it
+    p = sg.plan(dA, dB, semiring=1)
+    output = sg._output
+
+    def beside_least(q, nnz):
+        if q.ws.numel() > least:
+            raise torch.OutOfMemoryError("no room")
+        return output(q, nnz)
+
+    monkeypatch.setattr(sg, "_output", beside_least)
+    rp, nnz = sg.symbolic(p)
+    col, _ = sg.alloc_output(p, nnz)
+    sg.numeric(p, rp, col, None)
+    sg.check(p)
+    assert p.ws.numel() == least and right(rp, col)
