@@ -5,6 +5,8 @@
 #include <cstdio>
 #include <cstring>
 #include <atomic>
+#include <exception>
+#include <memory>
 #include <new>
 
 #include "plan.h"
@@ -158,10 +160,10 @@ static void set_chunks(Plan& P) {
 
 // Checks and records a batch of products; shared by spgemm_plan,
 // spgemm_batch_plan and spgemm_plan_device.
-spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
-                        const spgemm_opts* opts, void* stream, void* plan_ws, size_t plan_ws_bytes,
-                        bool device_sized, spgemm_plan_t* plan_out, const float* sizer_params,
-                        float sizer_margin) {
+static spgemm_status build_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
+                                const spgemm_opts* opts, void* stream, void* plan_ws,
+                                size_t plan_ws_bytes, bool device_sized, spgemm_plan_t* plan_out,
+                                const float* sizer_params, float sizer_margin) {
     g_last_error.clear();
     if (!plan_out) return fail(SPGEMM_ERR_INVALID_ARG, "plan output pointer is NULL");
     *plan_out = nullptr;
@@ -212,10 +214,7 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
 
     Plan* P = new (std::nothrow) Plan();
     if (!P) return fail(SPGEMM_ERR_OUT_OF_MEMORY, "host allocation of the plan failed");
-    auto bail = [&](spgemm_status s) {
-        delete P;
-        return s;
-    };
+    std::unique_ptr<Plan> owner(P);
     P->opts = o;
     P->stream = (cudaStream_t)stream;
     P->it = A[0].index_type;
@@ -312,7 +311,7 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
     std::memcpy(head.data() + ((unsigned char*)P->bb - P->pws), bb.data(),
                 (count + 1) * sizeof(long long));
     cudaError_t e = cudaMemcpyAsync(P->pws, head.data(), head.size(), cudaMemcpyHostToDevice, s);
-    if (e != cudaSuccess) return bail(cuda_fail(e, "plan: descriptor upload"));
+    if (e != cudaSuccess) return cuda_fail(e, "plan: descriptor upload");
 
     auto prepare = [&]() -> cudaError_t {
         const bool i32 = P->it == SPGEMM_INDEX_I32;
@@ -326,10 +325,10 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
         // sizes are upper bounds; the row analysis runs inside spgemm_execute
         P->max_dense_len = o.max_row_nnz ? o.max_row_nnz : 65536;
         e = prepare();
-        if (e != cudaSuccess) return bail(cuda_fail(e, "plan: numeric setup"));
+        if (e != cudaSuccess) return cuda_fail(e, "plan: numeric setup");
         e = cudaStreamSynchronize(s);  // the descriptor upload reads host buffers
-        if (e != cudaSuccess) return bail(cuda_fail(e, "plan: sync"));
-        *plan_out = P;
+        if (e != cudaSuccess) return cuda_fail(e, "plan: sync");
+        *plan_out = owner.release();
         return SPGEMM_OK;
     }
 
@@ -342,29 +341,29 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
                 e = P->it == SPGEMM_INDEX_I32 ? sg::launch_validate<int32_t>(B[p], err, P->sm_count, s)
                                               : sg::launch_validate<int64_t>(B[p], err, P->sm_count, s);
         }
-        if (e != cudaSuccess) return bail(cuda_fail(e, "plan: validate"));
+        if (e != cudaSuccess) return cuda_fail(e, "plan: validate");
         int herr = 0;
         e = cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, s);
         if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) return bail(cuda_fail(e, "plan: validate readback"));
+        if (e != cudaSuccess) return cuda_fail(e, "plan: validate readback");
         if (herr != 0)
-            return bail(fail(SPGEMM_ERR_INVALID_CSR, "invalid CSR input (%s)",
-                             herr == sg::kDevBadRowptr
-                                 ? "row pointers not monotone or out of range"
-                                 : "column index out of range, unsorted or duplicated"));
+            return fail(SPGEMM_ERR_INVALID_CSR, "invalid CSR input (%s)",
+                        herr == sg::kDevBadRowptr
+                            ? "row pointers not monotone or out of range"
+                            : "column index out of range, unsorted or duplicated");
     }
     e = P->it == SPGEMM_INDEX_I32 ? sg::launch_analyze<int32_t>(*P) : sg::launch_analyze<int64_t>(*P);
-    if (e != cudaSuccess) return bail(cuda_fail(e, "plan: analyze"));
+    if (e != cudaSuccess) return cuda_fail(e, "plan: analyze");
     e = sg::launch_binning(*P);
-    if (e != cudaSuccess) return bail(cuda_fail(e, "plan: binning"));
+    if (e != cudaSuccess) return cuda_fail(e, "plan: binning");
     sg::DevCounters h;
     e = cudaMemcpyAsync(&h, P->cnt, sizeof(h), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return bail(cuda_fail(e, "plan: readback"));
+    if (e != cudaSuccess) return cuda_fail(e, "plan: readback");
     if (h.unsupported)
-        return bail(fail(SPGEMM_ERR_NOT_SUPPORTED,
-                         "rows with more than %d products need n <= %lld columns (n = %lld)",
-                         P->dense_min, P->max_dense_n, P->max_n));
+        return fail(SPGEMM_ERR_NOT_SUPPORTED,
+                    "rows with more than %d products need n <= %lld columns (n = %lld)",
+                    P->dense_min, P->max_dense_n, P->max_n);
     long long acc = 0;
     for (int c = 0; c < sg::kNumClasses; ++c) {
         P->class_count[c] = h.class_count[c];
@@ -377,7 +376,7 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
     P->ndense = acc - P->class_off[sg::kClassDense0];
     P->max_dense_len = (long long)h.max_dense_len;
     e = prepare();
-    if (e != cudaSuccess) return bail(cuda_fail(e, "plan: numeric setup"));
+    if (e != cudaSuccess) return cuda_fail(e, "plan: numeric setup");
     {
         // A pattern's dense rows are in the bitmaps of the symbolic pass: they
         // are kept while they take no more than a byte per product (the columns
@@ -409,16 +408,29 @@ spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
                 set_chunks(*P);
                 e = cudaMemcpyAsync(P->d_descs, P->descs.data(), count * sizeof(sg::ProdDesc),
                                     cudaMemcpyHostToDevice, s);
-                if (e != cudaSuccess) return bail(cuda_fail(e, "plan: descriptor upload"));
+                if (e != cudaSuccess) return cuda_fail(e, "plan: descriptor upload");
             }
         }
         if (P->seg_log2 != 16) {
             e = sg::launch_class_offsets(*P);
-            if (e != cudaSuccess) return bail(cuda_fail(e, "plan: work units"));
+            if (e != cudaSuccess) return cuda_fail(e, "plan: work units");
         }
     }
-    *plan_out = P;
+    *plan_out = owner.release();
     return SPGEMM_OK;
+}
+
+// A host table that cannot be allocated is a status too.
+spgemm_status make_plan(int32_t count, const spgemm_csr* A, const spgemm_csr* B,
+                        const spgemm_opts* opts, void* stream, void* plan_ws, size_t plan_ws_bytes,
+                        bool device_sized, spgemm_plan_t* plan_out, const float* sizer_params,
+                        float sizer_margin) {
+    try {
+        return build_plan(count, A, B, opts, stream, plan_ws, plan_ws_bytes, device_sized, plan_out,
+                          sizer_params, sizer_margin);
+    } catch (const std::exception&) {
+        return fail(SPGEMM_ERR_OUT_OF_MEMORY, "host allocation of the plan failed");
+    }
 }
 
 spgemm_status check_ws(spgemm_plan_t P, void* ws, size_t ws_bytes) {

@@ -1,5 +1,6 @@
 // Non-template kernels: row binning, int64 exclusive scan, empty rows; and
 // their host launchers.
+#include <exception>
 #include <map>
 #include <tuple>
 
@@ -160,8 +161,11 @@ int occupancy_lookup(const void* kernel, int threads, size_t smem) {
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kernel, threads, smem) != cudaSuccess ||
         b < 1)
         return 1;   // an error is not remembered
-    if (known.size() >= 256) known.clear();
-    known[key] = b;
+    try {
+        if (known.size() >= 256) known.clear();
+        known[key] = b;
+    } catch (const std::exception&) {   // no room to remember it
+    }
     return b;
 }
 

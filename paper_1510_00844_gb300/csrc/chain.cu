@@ -3,6 +3,7 @@
 // one's output, run in one kernel launch (chain.cuh).
 #include <algorithm>
 #include <cstdio>
+#include <exception>
 #include <vector>
 
 #include "chain.h"
@@ -57,7 +58,7 @@ size_t spgemm_chain_workspace_size(int32_t nsteps) {
 
 spgemm_status spgemm_chain_create(int32_t nsteps, const spgemm_chain_step* steps,
                                   const spgemm_chain_opts* opts, void* chain_ws,
-                                  size_t chain_ws_bytes, spgemm_chain_t* chain_out) {
+                                  size_t chain_ws_bytes, spgemm_chain_t* chain_out) try {
     sg::set_last_error("");
     if (nsteps < 1 || !steps || !chain_out)
         return chain_fail(SPGEMM_ERR_INVALID_ARG, "need at least one step and a chain handle");
@@ -166,6 +167,8 @@ spgemm_status spgemm_chain_create(int32_t nsteps, const spgemm_chain_step* steps
     }
     *chain_out = C;
     return SPGEMM_OK;
+} catch (const std::exception&) {
+    return chain_fail(SPGEMM_ERR_OUT_OF_MEMORY, "host allocation of the chain failed");
 }
 
 spgemm_status spgemm_chain_launch(spgemm_chain_t C, void* stream) {

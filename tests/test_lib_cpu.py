@@ -138,3 +138,35 @@ def test_chain_argument_errors_need_no_gpu(lib):
     assert b"block_threads" in L.spgemm_last_error()
     assert L.spgemm_chain_create(1, steps, ctypes.byref(ok_opts), fake, need, ctypes.byref(h)) == 1
     assert b"plan" in L.spgemm_last_error()
+
+
+def test_failed_host_allocation_is_a_status(lib):
+    """A plan whose host tables do not fit the address space: a status, no
+    exception across the boundary (two million empty products, 50 MB left)."""
+    import subprocess
+    import sys
+    code = """
+import ctypes, resource, sys
+import numpy as np
+from paper_1510_00844_gb300 import build
+lib = ctypes.CDLL(build.LIB)
+count = 2_000_000
+# nrows, ncols, nnz, rowptr, rowend, col, val, {index type, value type}
+csr = np.zeros((count, 8), dtype=np.int64)
+csr[:, 3] = 8
+csr[:, 7] = 3 << 32
+plan = ctypes.c_void_p()
+size = lib.spgemm_batch_plan_workspace_size
+size.restype, size.argtypes = ctypes.c_size_t, [ctypes.c_int32, ctypes.c_void_p]
+need = size(count, csr.ctypes.data)
+pages = int(open('/proc/self/statm').read().split()[0]) * resource.getpagesize()
+resource.setrlimit(resource.RLIMIT_AS, (pages + 50_000_000, resource.RLIM_INFINITY))
+P = ctypes.c_void_p
+lib.spgemm_batch_plan.argtypes = [ctypes.c_int32, P, P, P, P, P, ctypes.c_size_t, P]
+st = lib.spgemm_batch_plan(count, csr.ctypes.data, csr.ctypes.data, None, None, 1 << 20, need,
+                           ctypes.byref(plan))
+assert plan.value is None
+sys.exit(st)
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT)
+    assert r.returncode == 4, (r.returncode, r.stderr[-500:])   # OUT_OF_MEMORY
