@@ -10,8 +10,9 @@
 //   scatter  (row, value) of every entry to its place in a scratch copy of
 //            A^T (arbitrary order inside a row; no further atomics);
 //   sort     every row of A^T from the scratch copy into the result, by
-//            original row index.  These are unique within a row, so the place
-//            of an entry is the number of smaller ones: rows of at most 8
+//            original row index.  The place of an entry is the number of
+//            smaller ones (and of equal ones before it in the scratch copy, for
+//            an A whose rows repeat a column): rows of at most 8
 //            entries take 8 lanes, of at most 32 a warp (both compare all
 //            pairs in registers), of at most 256 a warp's bitonic sort in
 //            shared memory; longer rows take a block and a bitmap of the
@@ -152,7 +153,10 @@ __global__ void __launch_bounds__(WARPS * 32)
                 if (x < Lr) v = vaS[ar + x];
             int place = 0;
 #pragma unroll
-            for (int y = 0; y < 8; ++y) place += __shfl_sync(kFull, key, y, 8) < key;
+            for (int y = 0; y < 8; ++y) {
+                const IT other = __shfl_sync(kFull, key, y, 8);
+                place += other < key || (other == key && y < x);
+            }
             if (x < Lr) {
                 ciT[ar + place] = key;
                 if constexpr (HV) vaT[ar + place] = v;
@@ -169,7 +173,10 @@ __global__ void __launch_bounds__(WARPS * 32)
                 if constexpr (HV)
                     if (lane < Lr) v = vaS[ar + lane];
                 int place = 0;
-                for (int y = 0; y < Lr; ++y) place += __shfl_sync(kFull, key, y) < key;
+                for (int y = 0; y < Lr; ++y) {
+                    const IT other = __shfl_sync(kFull, key, y);
+                    place += other < key || (other == key && y < lane);
+                }
                 if (lane < Lr) {
                     ciT[ar + place] = key;
                     if constexpr (HV) vaT[ar + place] = v;
@@ -303,6 +310,21 @@ __global__ void __launch_bounds__(THREADS)
             }
             __syncthreads();
             done += total;
+        }
+        if (done < L) {
+            // fewer rows than entries: a column is repeated in a row of A, and the
+            // bitmap holds one of the two.  Every entry counts those before it
+            for (long long x = threadIdx.x; x < L; x += THREADS) {
+                const IT key = ciS[a + x];
+                long long place = 0;
+                for (long long y = 0; y < L; ++y) {
+                    const IT other = ciS[a + y];
+                    place += other < key || (other == key && y < x);
+                }
+                ciT[a + place] = key;
+                if constexpr (HV) vaT[a + place] = vaS[a + x];
+            }
+            __syncthreads();
         }
     }
 }

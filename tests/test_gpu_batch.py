@@ -315,3 +315,33 @@ def test_row_pointer_scan_sizes(sg, n):
     R = oracle.transpose(A)
     assert np.array_equal(rp, R.rowptr) and np.array_equal(col, R.col)
     assert np.array_equal(val, R.val)
+
+
+@pytest.mark.parametrize("m", [400, 9000, 2_200_000])
+@pytest.mark.parametrize("index", [np.int32, np.int64])
+@pytest.mark.parametrize("value", ["u01_f64", "none"])
+def test_transpose_keeps_repeated_entries(sg, m, index, value):
+    """Rows of A that repeat a column, as a list of edges does before its sums are
+    formed: every entry of A is in A^T, at every column length at which the row
+    sorts change."""
+    rng = np.random.default_rng(m % 1000)
+    lens = [2, 3, 7, 8, 9, 31, 32, 33, 64, 255, 256, 257, 300, 1074, 1075, 3000, 8192, 8193, 9500]
+    rows, cols = [], []
+    for j, k in enumerate(lens):
+        some = rng.integers(0, m, max(1, k // 2))           # most rows twice and more
+        rows.append(np.concatenate([some, rng.choice(some, k - some.size)]))
+        cols.append(np.full(k, j))
+    rows, cols = np.concatenate(rows), np.concatenate(cols)
+    order = np.lexsort((cols, rows))
+    rows, cols = rows[order], cols[order]
+    A = inputs.CSR(m, len(lens), np.searchsorted(rows, np.arange(m + 1)).astype(np.int64),
+                   cols.astype(index), inputs.draw_values(rng, cols.size, value))
+    rp, col, val = sg.transpose(sg.to_device(A)).to_host()
+    assert np.array_equal(rp, np.concatenate([[0], np.cumsum(lens)]))
+    by_col = np.lexsort((rows, cols))
+    assert np.array_equal(col.astype(np.int64), rows[by_col])
+    if val is not None:
+        # the order of a pair's values is free
+        place = np.repeat(np.arange(len(lens)), lens)
+        assert np.array_equal(val[np.lexsort((val, col, place))],
+                              A.val[np.lexsort((A.val, rows, cols))])
