@@ -345,3 +345,49 @@ def test_transpose_keeps_repeated_entries(sg, m, index, value):
         place = np.repeat(np.arange(len(lens)), lens)
         assert np.array_equal(val[np.lexsort((val, col, place))],
                               A.val[np.lexsort((A.val, rows, cols))])
+
+
+def dense_batch(ns, value, index, seed):
+    """Products of 40 rows each, dense but for a few, of the given widths."""
+    rng = np.random.default_rng(seed)
+    out = []
+    for t, n in enumerate(ns):
+        l = 20 + 7 * t
+        A = inputs.random_csr(40, l, 0.8, seed + t, value=value, index_dtype=index, empty_rows=0.1)
+        # rows of B: half of the columns, the last among them; at most 20000
+        cols = [np.unique(np.append(rng.choice(n, min(n // 2, 20_000), replace=False), n - 1))
+                for _ in range(l)]
+        rp = np.concatenate([[0], np.cumsum([c.size for c in cols])]).astype(np.int64)
+        col = np.concatenate(cols).astype(index)
+        out.append((A, inputs.CSR(l, n, rp, col, inputs.draw_values(rng, col.size, value))))
+    return out
+
+
+@pytest.mark.parametrize("ns", [(40_000, 1500, 65_600, 33, 7001), (130, 4097, 128, 129),
+                                (262_145, 31, 900_000)])
+@pytest.mark.parametrize("index", [np.int32, np.int64])
+def test_batch_of_patterns_with_dense_rows(sg, ns, index):
+    """The bitmaps of a batch's dense rows have the widest product's words; each
+    product's columns come from its own."""
+    batch = dense_batch(ns, "none", index, 51)
+    As, Bs = [sg.to_device(a) for a, _ in batch], [sg.to_device(b) for _, b in batch]
+    p = sg.batch_plan(As, Bs, semiring=1)
+    assert p.info()["rows_dense"] > 0
+    for C, (A, B) in zip(sg.batch_spgemm(As, Bs, semiring=1, verify=True), batch):
+        assert_pattern_equal(C, oracle.spgemm(A, B, semiring="or_and"))
+
+
+@pytest.mark.parametrize("ns,width", [((130, 700, 3001), 256), ((130, 2048, 1025), 128),
+                                      ((2049, 60), 256), ((3001, 16_385), 1024),
+                                      ((130, 262_145, 16_384), 2048)])
+def test_batch_over_the_limits_of_chunk_widths(sg, ns, width):
+    """Narrow and wide products in one batch: the widest sets the chunks of all,
+    down to a product of one chunk beside one of hundreds."""
+    batch = dense_batch(ns, "u01_f64", np.int32, 61)
+    As, Bs = [sg.to_device(a) for a, _ in batch], [sg.to_device(b) for _, b in batch]
+    info = sg.batch_plan(As, Bs).info()
+    assert info["rows_dense"] > 0 and info["chunk_width"] == width
+    for C, (A, B) in zip(sg.batch_spgemm(As, Bs, verify=True), batch):
+        R = oracle.spgemm(A, B)
+        assert_pattern_equal(C, R)
+        assert np.array_equal(C.to_host()[2], R.val)

@@ -25,6 +25,14 @@ def run(sg, A, B, semiring=0, checked=True):
     return sg.spgemm(dA, dB, semiring=semiring, checked=checked, verify=True)
 
 
+SEMIRING = {0: "plus_times", 1: "or_and", 2: "min_plus", 3: "min_select2nd"}
+
+# value type, semiring and index type of the row-size tests
+VALUE_FORMS = [("u01_f64", 0, np.int32), ("int", 0, np.int32), ("none", 1, np.int32),
+               ("u01_f64", 0, np.int64), ("none", 1, np.int64), ("u01_f64", 2, np.int32),
+               ("int", 2, np.int64), ("u01_f64", 3, np.int64), ("int", 3, np.int32)]
+
+
 def check_product(sg, A, B, dtype="f64"):
     C = run(sg, A, B)
     R = oracle.spgemm(A, B)
@@ -449,8 +457,8 @@ def test_merge_more_long_rows_than_listed(sg):
 
 
 @pytest.mark.parametrize("n", [900, (1 << 25) - 1, 1 << 25])
-@pytest.mark.parametrize("value", ["u01_f64", "int", "none"])
-def test_rows_of_33_to_128_products(sg, n, value):
+@pytest.mark.parametrize("value,sr,index", VALUE_FORMS)
+def test_rows_of_33_to_128_products(sg, n, value, sr, index):
     """Rows around the bounds of the register sort (64 and 128 products) with
     all columns distinct, all equal and mixed, over many A entries and over
     few, the last column among them; n = 2^25 is the first width whose rows
@@ -464,7 +472,7 @@ def test_rows_of_33_to_128_products(sg, n, value):
             c = rng.choice(min(n, 5000), k, replace=False) if s == "spread" else np.arange(k)
             cols.append(np.sort(c if s != "right" else n - k + c))
     rp = np.concatenate([[0], np.cumsum([c.size for c in cols])]).astype(np.int64)
-    col = np.concatenate(cols).astype(np.int32)
+    col = np.concatenate(cols).astype(index)
     B = inputs.CSR(len(cols), n, rp, col, inputs.draw_values(rng, col.size, value))
     size = np.diff(rp)
     rows = []
@@ -477,20 +485,23 @@ def test_rows_of_33_to_128_products(sg, n, value):
                     left -= size[k]
             rows.append(np.sort(pick))
     rpA = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
-    colA = np.concatenate(rows).astype(np.int32)
+    colA = np.concatenate(rows).astype(index)
     A = inputs.CSR(len(rows), len(cols), rpA, colA, inputs.draw_values(rng, colA.size, value))
-    sr = 1 if value == "none" else 0
     C = run(sg, A, B, semiring=sr)
-    R = oracle.spgemm(A, B, semiring="or_and" if sr else "plus_times")
+    R = oracle.spgemm(A, B, semiring=SEMIRING[sr])
     assert_pattern_equal(C, R)
     if value != "none":
         assert np.array_equal(C.to_host()[2], R.val)
 
 
-@pytest.mark.parametrize("n,value", [(2000, "u01_f64"), (16384, "none"), (16385, "u11_f32"),
-                                     (32768, "int"), (32769, "u01_f64"), (262144, "u01_f64"),
-                                     (262144, "none"), (262145, "int")])
-def test_rows_of_129_to_1024_products(sg, n, value):
+@pytest.mark.parametrize("n,value,sr,index",
+                         [(2000, "u01_f64", 0, np.int32), (16384, "none", 1, np.int32),
+                          (16385, "u11_f32", 0, np.int32), (32768, "int", 0, np.int32),
+                          (32769, "u01_f64", 0, np.int32), (262144, "u01_f64", 0, np.int32),
+                          (262144, "none", 1, np.int32), (262145, "int", 0, np.int32)]
+                         + [(n, *form) for n in (2000, 32768, 262144, 262145)
+                            for form in VALUE_FORMS[3:]])
+def test_rows_of_129_to_1024_products(sg, n, value, sr, index):
     """Rows at the edges of the bitmap-ranked bins, on both sides of the widths
     up to which they are ranked: all columns distinct, every column hit by many
     A entries, and single products over a thousand A entries between empty
@@ -510,7 +521,7 @@ def test_rows_of_129_to_1024_products(sg, n, value):
     cols = [cols[t] for t in order]
     size = np.array([c.size for c in cols])
     B = inputs.CSR(len(cols), n, np.concatenate([[0], np.cumsum(size)]).astype(np.int64),
-                   np.concatenate(cols).astype(np.int32),
+                   np.concatenate(cols).astype(index),
                    inputs.draw_values(rng, int(size.sum()), value))
     rows = []
     for target in [128, 129, 130, 511, 512, 513, 1000, 1023, 1024, 1025]:
@@ -524,12 +535,11 @@ def test_rows_of_129_to_1024_products(sg, n, value):
                     if left == 0:
                         break
                 rows.append(np.sort(pick))
-    colA = np.concatenate(rows).astype(np.int32)
+    colA = np.concatenate(rows).astype(index)
     rpA = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
     A = inputs.CSR(len(rows), len(cols), rpA, colA, inputs.draw_values(rng, colA.size, value))
-    sr = 1 if value == "none" else 0
     C = run(sg, A, B, semiring=sr)
-    R = oracle.spgemm(A, B, semiring="or_and" if sr else "plus_times")
+    R = oracle.spgemm(A, B, semiring=SEMIRING[sr])
     assert_pattern_equal(C, R)
     if value == "u11_f32":
         assert_values_close(C, R, A, B, "f32")
@@ -537,16 +547,19 @@ def test_rows_of_129_to_1024_products(sg, n, value):
         assert np.array_equal(C.to_host()[2], R.val)
 
 
-@pytest.mark.parametrize("n,l,value", [(130, 300, "u01_f64"), (700, 200, "none"),
-                                       (1025, 150, "u11_f32"), (2047, 120, "int"),
-                                       (3001, 100, "u01_f64"), (16500, 60, "u01_f64")])
-def test_dense_rows_in_narrow_chunks(sg, n, l, value):
+@pytest.mark.parametrize("n,l,value,width", [(130, 300, "u01_f64", 128), (700, 200, "none", 128),
+                                             (1025, 150, "u11_f32", 128), (2047, 120, "int", 128),
+                                             (3001, 100, "u01_f64", 256),
+                                             (16500, 60, "u01_f64", 1024)])
+def test_dense_rows_in_narrow_chunks(sg, n, l, value, width):
     """Few columns, long rows: the chunks of the dense rows are narrowed (down to
     128 columns) so that a row makes several work units; 16500 columns keep
     the full width for float64.  Plain and learned sizing."""
     A = inputs.random_csr(90, l, 0.6, 31 + n, value=value, index_dtype=np.int32)
     B = inputs.random_csr(l, n, 0.5, 32 + n, value=value, index_dtype=np.int32, empty_rows=0.1)
     sr = 1 if value == "none" else 0
+    info = sg.plan(sg.to_device(A), sg.to_device(B), semiring=sr).info()
+    assert info["rows_dense"] > 0 and info["chunk_width"] == width
     C = run(sg, A, B, semiring=sr)
     R = oracle.spgemm(A, B, semiring="or_and" if sr else "plus_times")
     assert_pattern_equal(C, R)
@@ -590,9 +603,9 @@ def test_pattern_of_dense_rows(sg, n, rows, l, density, index):
         assert np.array_equal(col.cpu().numpy().astype(np.int64), R.col)
 
 
-@pytest.mark.parametrize("value", ["u01_f64", "u11_f32", "int", "none"])
+@pytest.mark.parametrize("value,sr,index", VALUE_FORMS + [("u11_f32", 0, np.int32)])
 @pytest.mark.parametrize("n", [700, 2**23 - 1, 2**23])
-def test_rows_of_129_to_512_products_sorted(sg, n, value):
+def test_rows_of_129_to_512_products_sorted(sg, n, value, sr, index):
     """Rows on both sides of eight and sixteen keys per lane, with distinct
     columns, with columns that most B rows share and with the last column, on
     both sides of the width up to which a warp sorts them."""
@@ -604,7 +617,7 @@ def test_rows_of_129_to_512_products_sorted(sg, n, value):
         cols.append(np.sort(c))
     size = np.array([c.size for c in cols])
     B = inputs.CSR(len(cols), n, np.concatenate([[0], np.cumsum(size)]).astype(np.int64),
-                   np.concatenate(cols).astype(np.int32),
+                   np.concatenate(cols).astype(index),
                    inputs.draw_values(rng, int(size.sum()), value))
     rows = []
     for target in [129, 160, 161, 255, 256, 257, 288, 289, 511, 512]:
@@ -615,12 +628,11 @@ def test_rows_of_129_to_512_products_sorted(sg, n, value):
                     pick.append(k)
                     left -= size[k]
             rows.append(np.sort(pick))
-    colA = np.concatenate(rows).astype(np.int32)
+    colA = np.concatenate(rows).astype(index)
     rpA = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int64)
     A = inputs.CSR(len(rows), len(cols), rpA, colA, inputs.draw_values(rng, colA.size, value))
-    sr = 1 if value == "none" else 0
     C = run(sg, A, B, semiring=sr)
-    R = oracle.spgemm(A, B, semiring="or_and" if sr else "plus_times")
+    R = oracle.spgemm(A, B, semiring=SEMIRING[sr])
     assert_pattern_equal(C, R)
     if value == "u11_f32":
         assert_values_close(C, R, A, B, "f32")
