@@ -297,10 +297,10 @@ def _timed(torch, fn, reps):
 def merge_roofline(sg, torch, dA, c=4, reps=3):
     """The multiway merge alone on the 4 k-slice partials of the product
     (count + scan + numeric, then the numeric pass by itself), the default
-    form (reported as "windows") against lists staged in shared memory by
-    bulk asynchronous copies.  Algorithmic bytes of the numeric pass: every partial entry read
-    once and every entry of C written once (index + value each), plus the c
-    partial row-pointer arrays and rowptr(C)."""
+    form against lists staged in shared memory by bulk asynchronous copies.
+    Algorithmic bytes of the numeric pass: every partial entry read once and
+    every entry of C written once (index + value each), plus the c partial
+    row-pointer arrays and rowptr(C)."""
     _, parts = sg.spgemm_kslice(dA, dA, c)
     torch.cuda.synchronize()
     m = dA.nrows
@@ -314,7 +314,7 @@ def merge_roofline(sg, torch, dA, c=4, reps=3):
     stream = torch.cuda.current_stream()
     hbm, _ = peaks()
     res = {"partial_entries": nparts, "nnz_C": int(nnz), "algorithmic_bytes": int(nbytes)}
-    for name, staged in (("windows", False), ("staged", True)):
+    for name, staged in (("default", False), ("staged", True)):
         sg.merge_numeric(parts, ws, rowptrC, colC, valC, staged=staged)
         sg.merge_check(ws)
         ms = []

@@ -1109,10 +1109,10 @@ __global__ void __launch_bounds__(MAXT, MINB) symbolic_dense_kernel(const ProdDe
 // chunks; the chunks' counts give its place in C(i,:).  A lane takes four words
 // and puts their bits' offsets into the warp's stage, highest first (one
 // instruction of the slow pipe per bit), so that the stores to C are coalesced.
-// What bounds it: DRAM traffic (the bitmaps once, C once) in part and the bit
-// loops; sweeping the products of every row again took as long as their symbolic
-// pass.  R-MAT, 100003 vertices (233 M columns): sweep 1.82 ms, a word per lane
-// and a scan for each 0.63 ms, four 0.59 ms; loading a step ahead 0.60 ms.
+// What bounds it: instructions, the bit loops (issue 75 % active, DRAM 28 % of
+// its peak); sweeping the products of every row again took as long as their
+// symbolic pass.  R-MAT, 100003 vertices (233 M columns): sweep 1.82 ms, a word
+// per lane and a scan for each 0.63 ms, four 0.59 ms; loading a step ahead 0.60 ms.
 constexpr int kColStage = 512;   // of the 4096 columns of 128 words
 template <class IT>
 __global__ void __launch_bounds__(256, 8)
@@ -1613,7 +1613,8 @@ struct __align__(16) DenseRun {
 // sorted.  The first product of every place (the smallest f, by atomicMin)
 // stores its value; the others, few in a sparse row, are listed in ascending f
 // and added by one warp in that order.
-// What bounds it: instructions, at 24 to 28 warps per SM.  A warp with a table
+// What bounds it: instructions and shared memory (numeric float32: issue 57 %, L1
+// 74 %), at 24 to 36 warps per SM.  A warp with a table
 // per row (25 KB for float64) held 12 warps and took 9.7 instructions per
 // product: 64 uneven Erdos-Renyi products in float32 (up to 65536 columns),
 // rows of 513 to 1024 products 6.25 -> 2.34 ms, their counts 1.45 -> 0.91 ms.

@@ -109,9 +109,11 @@ cudaError_t launch_kslice_bounds(const spgemm_csr& A, int c, int64_t* bounds, in
 // Erdos-Renyi squares, float64, table and bitmap in us: 30 per column (bin 3),
 // numeric 352 and 57 at 8192 columns, 1949 and 445 at 65536, 4194 and 1381 at
 // 131072, 8464 and 5384 at 262144; counts 53 and 21, 327 and 148, 623 and 321,
-// 1214 and 935; 16 per column (bin 2), numeric 60 and 42 at 8192, 187 and 159 at
-// 32768, 350 and 335 at 65536 (float32 288 and 303; uneven batches up to 65536
-// columns 2540 and 3060); counts 33 and 29 at 16384, 56 and 60 at 32768.
+// 1214 and 935; 16 per column (bin 2), counts 33 and 29 at 16384, 56 and 60 at
+// 32768; numeric, which only predicted slots take (the others are sorted, see
+// sort_bin), 97 and 42 at 8192, 302 and 161 at 32768, in float32 83 and 38, 254
+// and 143; with exact slots the two met at 65536 columns (350 and 335; float32 288
+// and 303).
 inline bool rank_bin(const Plan& P, int bin, bool count) {
     return P.max_n <= rank_max_n(bin, count);
 }

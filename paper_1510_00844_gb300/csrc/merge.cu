@@ -16,8 +16,9 @@
 // column segments: a power-law graph's longest row holds more entries than a
 // warp should add while the others have finished.
 //
-// What bounds it: the latency of a chunk's few dependent steps (columns, map,
-// values) at 20 warps per SM, then DRAM.  The sweep of 1024-column chunks that
+// What bounds it: the count, instructions (issue 82 % active); the numeric pass,
+// instructions and the latency of a chunk's few dependent steps (columns, map,
+// values) at 20 warps per SM (issue 53 %, DRAM 21 %).  The sweep of 1024-column chunks that
 // this replaces met few entries per chunk on rows of ordinary length and left
 // the longest rows to single warps.  Before and now: four lists of 100003-vertex
 // R-MAT graphs (3.3 GB read and written) 5.70 and 2.80 ms; the four partial
